@@ -16,11 +16,15 @@
 // PL_f = Phi Mref^{-1} E_f the lift of face f. Three kernels per chunk of elements:
 //   k_pointwise  one thread per quadrature point: fluxes and exact pointwise Jacobians
 //                by forward-mode dual numbers, pre-contracted with weights and Jinv;
-//   k_assemble   one CTA per element: quadrature contractions into A', B', C', D', R;
+//   k_assemble   one CTA per element: quadrature contractions into A', B', C', D', R
+//                (element_fp64.cuh);
 //   k_condense   one CTA per element: LU with partial pivoting of A' in shared memory,
 //                triangular solves for X and y, Schur products for S and g.
 #pragma once
+#include <type_traits>
+
 #include "dfloat.cuh"
+#include "element_fp64.cuh"
 #include "hdg_device.cuh"
 
 namespace hdg {
@@ -121,6 +125,31 @@ HDG_DEVI void volume_point_state(int g, const DevTables& T, const double (*z)[C:
 HDG_DEVI void put(double* p, int i, double v) { p[i] = v; }
 HDG_DEVI void put(df2* p, int i, double v) { p[i] = df_from(v); }
 
+// Point tensors of one point: the FP64 form stores them [quantity][point] (element_fp64.cuh: the
+// contractions read one quantity over the points), the mixed form [point][quantity].
+template <class OutT, int NPT>
+struct PtOut {
+  static constexpr int S = std::is_same<OutT, double>::value ? NPT : 1;
+  OutT* p;
+  HDG_DEVI PtOut operator+(int i) const { return {p + i * S}; }
+};
+template <class OutT, int NPT>
+HDG_DEVI void put(const PtOut<OutT, NPT>& o, int i, double v) {
+  put(o.p, i * PtOut<OutT, NPT>::S, v);
+}
+
+// row r of Jinv, or the sum of the rows (r = D)
+template <int D>
+HDG_DEVI void jinv_row(const double* Jinv, int r, double* out) {
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < D; ++q) s += Jinv[q * D + k];
+    out[k] = r < D ? Jinv[r * D + k] : s;
+  }
+}
+
 // The values of sigma(vhat) = d(sigma (v - vhat))/dv at one face point, [row][column]:
 // lambda_max A0 (Eq. sLxF) from the wave speed and u(vhat)'s derivatives, or |A_n| A0 (Eq. symStab)
 // as a table.
@@ -181,12 +210,9 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
       for (int i = 0; i < M; ++i)
         for (int j = 0; j < D; ++j) F[i][j] = F[i][j] + Gv[i][j];
     }
-    OutT* out = reinterpret_cast<OutT*>(a.ptv) + (le * NG + g) * C::PT_VOL;
-    OutT* MU = out;
-    OutT* FR = MU + M;
-    OutT* T0 = FR + D * M;
-    OutT* T1 = T0 + M * M;
-    OutT* T2 = T1 + D * M * M;
+    using Pt = PtOut<OutT, NG>;
+    const Pt MU{reinterpret_cast<OutT*>(a.ptv) + (Pt::S == 1 ? (le * NG + g) * C::PT_VOL : le * NG * C::PT_VOL + g)};
+    const Pt FR = MU + M, T0 = FR + D * M, T1 = T0 + M * M, T2 = T1 + D * M * M;
     for (int i = 0; i < M; ++i) {
       put(MU, i, W * a.mass_coef * u[i].v);
       for (int l = 0; l < M; ++l) put(T0, i * M + l, W * a.mass_coef * u[i].d[l]);
@@ -206,11 +232,22 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
       // dG/dq contracted with the rows of Jinv (G is linear in q)
       const ViscFactors<D> vf = visc_factors<D>(v);
       const PhysParams pv = visc_params_at(ph, v[M - 1]);
+      if constexpr (Pt::S > 1) {  // on both sides
 #pragma unroll 1
-      for (int r = 0; r < D; ++r)
-        visc_jac_dir<D>(vf, Jinv + r * D, pv, [&](int i, int l, int k, double val) {
-          put(T2, ((r * M + i) * M + l) * D + k, -W * val);
-        });
+        for (int rr = 0; rr < D * (D + 1); ++rr) {
+          double c2[D];
+          jinv_row<D>(Jinv, rr % (D + 1), c2);
+          visc_jac_pair<D>(vf, Jinv + rr / (D + 1) * D, c2, pv, [&](int i, int l, double val) {
+            put(T2, (rr * (M - 1) + i - 1) * (M - 1) + l - 1, -W * val);
+          });
+        }
+      } else {
+#pragma unroll 1
+        for (int r = 0; r < D; ++r)
+          visc_jac_dir<D>(vf, Jinv + r * D, pv, [&](int i, int l, int k, double val) {
+            put(T2, ((r * M + i) * M + l) * D + k, -W * val);
+          });
+      }
     }
   } else if (tid < NG + NF * NGF) {
     const int f = (tid - NG) / NGF;
@@ -305,11 +342,11 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
     prim_of_v<D>(vd, ph.gamma, rv, velv, pv);
     cons_and_flux<D>(rv, velv, pv, ph.gamma, (Dual<M>*)nullptr, Fv);
     bad = bad || !(rv.v > 0.0) || !(pv.v > 0.0);
-    OutT* out = reinterpret_cast<OutT*>(a.ptf) + ((le * NF + f) * NGF + gf) * C::PT_FACE;
-    OutT* HF = out;
-    OutT* U0 = HF + M;
-    OutT* U1 = U0 + M * M;
-    OutT* U2 = U1 + M * M;
+    using Pt = PtOut<OutT, NF * NGF>;
+    const int pf = f * NGF + gf;
+    const Pt HF{reinterpret_cast<OutT*>(a.ptf) +
+                (Pt::S == 1 ? (le * NF * NGF + pf) * C::PT_FACE : le * NF * NGF * C::PT_FACE + pf)};
+    const Pt U0 = HF + M, U1 = U0 + M * M, U2 = U1 + M * M;
     Dual<M> gn[M];  // ghat = G(v, q) . n (Eq. numericalFluxNS_1): value and d/dv
     for (int i = 0; i < M; ++i) gn[i] = vd[0] * 0.0;
     if (C::VISC && ph.gflux == 1) {
@@ -330,8 +367,19 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
     if (C::VISC) {  // dG/dq contracted with the normal, at the state the viscous flux uses
       const double* vs = ph.gflux == 1 ? v : vh;
       const ViscFactors<D> vf = visc_factors<D>(vs);
-      visc_jac_dir<D>(vf, n, visc_params_at(ph, vs[M - 1]),
-                      [&](int i, int l, int k, double val) { put(U2, (i * M + l) * D + k, Wf * val); });
+      const PhysParams pvs = visc_params_at(ph, vs[M - 1]);
+      if constexpr (Pt::S > 1) {
+#pragma unroll 1
+        for (int r = 0; r <= D; ++r) {
+          double c2[D];
+          jinv_row<D>(Jinv, r, c2);
+          visc_jac_pair<D>(vf, n, c2, pvs, [&](int i, int l, double val) {
+            put(U2, (r * (M - 1) + i - 1) * (M - 1) + l - 1, Wf * val);
+          });
+        }
+      } else {
+        visc_jac_dir<D>(vf, n, pvs, [&](int i, int l, int k, double val) { put(U2, (i * M + l) * D + k, Wf * val); });
+      }
     }
   }
   if (bad) atomicOr(a.status + e, HDG_STATUS_NONPHYSICAL);
@@ -348,370 +396,109 @@ void launch_pointwise(const AssembleArgs& a, const DevTables& T, const PhysParam
 }
 
 // ------------------------------------------------------------------------------------
-// k_assemble
+// k_assemble: one CTA per element (element_blocks), several per SM
 // ------------------------------------------------------------------------------------
 template <class C>
-struct AsmSmem {
-  static constexpr int GT = C::NG < 64 ? C::NG : 64;  // volume points per tile
-  static constexpr int RB = C::NR * GT * C::NZ;
-  static constexpr int RBF = C::NRF * C::NGF * C::NZ;
-  static constexpr int RBMAX = RB > RBF ? RB : RBF;
-  static constexpr int ZS = C::NP * GT * C::NR;
-  static constexpr int ZSF = C::NFN * C::NGF * C::NRF;
-  static constexpr int ZSMAX = ZS > ZSF ? ZS : ZSF;
-  static constexpr size_t bytes =
-      sizeof(double) * (RBMAX + ZSMAX + C::NZ * C::M + C::GEO + C::NV + C::NT);
+struct UniformDims {
+  static constexpr int pad(int n) { return (n + 1) / 2 * 2; }
+  static constexpr int NP = C::NP, NG = C::NG, NGF = C::NGF, NTN = C::NF * C::NFN, NV = C::NV, NT = C::NT;
+  static constexpr int NPs = pad(C::NP), NZs = NPs + C::NF * pad(C::NFN);
 };
 
 template <class C>
-__global__ void __launch_bounds__(256) k_assemble(AssembleArgs a, DevTables T) {
-  constexpr int D = C::D, M = C::M, NP = C::NP, NFN = C::NFN, NF = C::NF, NG = C::NG, NGF = C::NGF;
-  constexpr int NZ = C::NZ, NV = C::NV, NT = C::NT, NR = C::NR, NRF = C::NRF;
-  using SM = AsmSmem<C>;
-  constexpr int GT = SM::GT;
-  extern __shared__ double smem[];
-  double* Rb = smem;
-  double* Zs = Rb + SM::RBMAX;
-  double(*z)[M] = reinterpret_cast<double(*)[M]>(Zs + SM::ZSMAX);
-  double* G = Zs + SM::ZSMAX + NZ * M;
-  double* Rv = G + C::GEO;
-  double* Rt = Rv + NV;
+struct AsmSmem {
+  static constexpr int NTH = C::D == 3 && C::P >= 2 ? 256 : 128;
+  // tiles of one operator: A' and one face's block of B'
+  static constexpr int TILES = UniformDims<C>::NPs / 2 * (UniformDims<C>::NPs / 2 + (C::VISC ? (C::NFN + 1) / 2 : 0));
+  static constexpr int NRD = (TILES + NTH - 1) / NTH;
+  static constexpr int MINB = NTH == 256 ? 3 : 5;  // registers: 80 a thread
+  static constexpr int H = C::NF * C::NGF * UniformDims<C>::NZs, Z = 2 * C::NG * UniformDims<C>::NPs;
+  static constexpr size_t bytes = sizeof(double) * (UniformDims<C>::NTN * UniformDims<C>::NZs + (H > Z ? H : Z));
+};
+
+// the reference operators of an element of one degree, filled in by one thread
+template <class C>
+HDG_DEVI void uniform_tables(const DevTables& T, ElemTables<C::D>& E) {
+  constexpr int NF = C::NF, NFN = C::NFN, NG = C::NG, NGF = C::NGF;
+  E.Phi = T.Phi;
+  E.dPhi = T.dPhi;
+  E.dR = T.dR;
+  E.PhiF = T.PhiF;
+  E.dRF = T.dRF;
+  E.nodepos = T.nodepos;
+  for (int f = 0; f < NF; ++f) {
+    E.Psi[f] = T.Psi + f * NGF * NFN;
+    E.PL[f] = T.PL + f * NG * NFN;
+    E.PLF[f] = T.PLF + f * NGF * NFN;
+    E.sPLF[f] = NF * NGF * NFN;
+    E.Tr[f] = nullptr;
+    E.nq[f] = NFN;
+  }
+  for (int f = 0; f <= NF; ++f) {
+    E.off[f] = f * NFN;
+    E.offp[f] = f * ((NFN + 1) / 2 * 2);
+  }
+}
+
+template <class C>
+__global__ void __launch_bounds__(AsmSmem<C>::NTH, AsmSmem<C>::MINB) k_assemble(AssembleArgs a, DevTables T) {
+  constexpr int D = C::D, NF = C::NF, NG = C::NG, NGF = C::NGF, NV = C::NV, NT = C::NT, NTH = AsmSmem<C>::NTH;
+  extern __shared__ __align__(16) double smem[];
+  __shared__ ElemTables<D> E;
   const int64_t le = blockIdx.x;
   const int64_t e = a.e0 + le;
   if (skip_element(a, e)) return;
-  const int tid = threadIdx.x, nth = blockDim.x;
-  load_element<C>(a, e, z, G);
+  if (threadIdx.x == 0) uniform_tables<C>(T, E);
   __syncthreads();
-  const double* Jinv = G;
-  const double detJ = G[D * D];
-  double* Ap = a.Ap + le * NV * NV;
-  double* Cp = a.Cp + le * NT * NV;
-  double* Bp = a.recov + e * (int64_t)(NV * NT + NV);
-  double* Dp = a.S + e * (int64_t)NT * NT;
   const double* ptv = a.ptv + le * NG * C::PT_VOL;
   const double* ptf = a.ptf + le * NF * NGF * C::PT_FACE;
-
-  // residual R_v, volume part
-  for (int t = tid; t < NV; t += nth) {
-    int an = t / M, i = t % M;
-    double s = a.hist ? -a.hist[e * NV + t] : 0.0;
-    for (int g = 0; g < NG; ++g) {
-      const double* P = ptv + g * C::PT_VOL;
-      s += T.Phi[g * NP + an] * P[i];
-      for (int r = 0; r < D; ++r) s += T.dPhi[(r * NG + g) * NP + an] * P[M + r * M + i];
-    }
-    Rv[t] = s;
-  }
-
-  // ---------------- volume contractions ----------------
-  for (int g0 = 0; g0 < NG; g0 += GT) {
-    const int ng = (NG - g0) < GT ? (NG - g0) : GT;
-    __syncthreads();
-    // right operators Rb[beta][gg][j]
-    for (int t = tid; t < NR * GT * NZ; t += nth) {
-      int beta = t / (GT * NZ), gg = (t / NZ) % GT, j = t % NZ;
-      double val = 0.0;
-      if (gg < ng) {
-        int g = g0 + gg;
-        if (beta == 0) {
-          val = j < NP ? T.Phi[g * NP + j] : 0.0;
-        } else {
-          int k = beta - 1;
-          if (j < NP) {
-            for (int r = 0; r < D; ++r) val += Jinv[r * D + k] * T.dPhi[(r * NG + g) * NP + j];
-            for (int f = 0; f < NF; ++f) {
-              int c = T.nodepos[f * NP + j];
-              if (c >= 0) {
-                const double* Gf = G + D * D + 1 + f * (D + 1);
-                val -= Gf[k] * (Gf[D] / detJ) * T.PL[(f * NG + g) * NFN + c];
-              }
-            }
-          } else {
-            int f = (j - NP) / NFN, c = (j - NP) % NFN;
-            const double* Gf = G + D * D + 1 + f * (D + 1);
-            val = Gf[k] * (Gf[D] / detJ) * T.PL[(f * NG + g) * NFN + c];
-          }
-        }
-      }
-      Rb[t] = val;
-    }
-    for (int il = 0; il < M * M; ++il) {
-      const int i = il / M, l = il % M;
-      __syncthreads();
-      // Zs[a][gg][beta] = sum_alpha L_alpha(g, a) C^{il}_{alpha beta}(g)
-      for (int t = tid; t < NP * GT * NR; t += nth) {
-        int an = t / (GT * NR), gg = (t / NR) % GT, beta = t % NR;
-        double val = 0.0;
-        if (gg < ng) {
-          int g = g0 + gg;
-          const double* P = ptv + g * C::PT_VOL;
-          const double* T0 = P + M + D * M;
-          const double* T1 = T0 + M * M;
-          const double* T2 = T1 + D * M * M;
-          if (beta == 0) {
-            val = T.Phi[g * NP + an] * T0[i * M + l];
-            for (int r = 0; r < D; ++r) val += T.dPhi[(r * NG + g) * NP + an] * T1[(r * M + i) * M + l];
-          } else {
-            int k = beta - 1;
-            for (int r = 0; r < D; ++r)
-              val += T.dPhi[(r * NG + g) * NP + an] * T2[((r * M + i) * M + l) * D + k];
-          }
-        }
-        Zs[t] = val;
-      }
-      __syncthreads();
-      for (int t = tid; t < NP * NZ; t += nth) {
-        int an = t / NZ, j = t % NZ;
-        const int b0 = j < NP ? 0 : 1;
-        double acc = 0.0;
-        for (int gg = 0; gg < ng; ++gg)
-          for (int beta = b0; beta < NR; ++beta) acc += Zs[(an * GT + gg) * NR + beta] * Rb[(beta * GT + gg) * NZ + j];
-        int row = an * M + i;
-        if (j < NP) {
-          double* dst = Ap + row * NV + j * M + l;
-          *dst = (g0 == 0) ? acc : *dst + acc;
-        } else {
-          double* dst = Bp + row * NT + (j - NP) * M + l;
-          *dst = (g0 == 0) ? acc : *dst + acc;
-        }
-      }
-    }
-  }
-
-  // ---------------- face contractions ----------------
-  for (int f = 0; f < NF; ++f) {
-    __syncthreads();
-    const double* Gf = G + D * D + 1 + f * (D + 1);
-    for (int t = tid; t < NRF * NGF * NZ; t += nth) {
-      int beta = t / (NGF * NZ), gf = (t / NZ) % NGF, j = t % NZ;
-      const double* phif = T.PhiF + (f * NGF + gf) * NP;
-      double val = 0.0;
-      if (beta == 0) {
-        val = j < NP ? phif[j] : 0.0;
-      } else if (beta == 1) {
-        if (j >= NP && (j - NP) / NFN == f) val = phif[T.fnodes[f * NFN + (j - NP) % NFN]];
-      } else {
-        int k = beta - 2;
-        if (j < NP) {
-          for (int r = 0; r < D; ++r) val += Jinv[r * D + k] * T.dPhiF[((f * D + r) * NGF + gf) * NP + j];
-          for (int fl = 0; fl < NF; ++fl) {
-            int c = T.nodepos[fl * NP + j];
-            if (c >= 0) {
-              const double* Gl = G + D * D + 1 + fl * (D + 1);
-              val -= Gl[k] * (Gl[D] / detJ) * T.PLF[((f * NF + fl) * NGF + gf) * NFN + c];
-            }
-          }
-        } else {
-          int fl = (j - NP) / NFN, c = (j - NP) % NFN;
-          const double* Gl = G + D * D + 1 + fl * (D + 1);
-          val = Gl[k] * (Gl[D] / detJ) * T.PLF[((f * NF + fl) * NGF + gf) * NFN + c];
-        }
-      }
-      Rb[t] = val;
-    }
-    (void)Gf;
-    // residual: face contribution
-    __syncthreads();
-    for (int t = tid; t < NFN * M; t += nth) {
-      int c = t / M, i = t % M;
-      double s = 0.0;
-      for (int gf = 0; gf < NGF; ++gf) {
-        double psi = T.PhiF[(f * NGF + gf) * NP + T.fnodes[f * NFN + c]];
-        s += psi * ptf[(f * NGF + gf) * C::PT_FACE + i];
-      }
-      Rv[T.fnodes[f * NFN + c] * M + i] += s;
-      Rt[(f * NFN + c) * M + i] = s;
-    }
-    for (int il = 0; il < M * M; ++il) {
-      const int i = il / M, l = il % M;
-      __syncthreads();
-      for (int t = tid; t < NFN * NGF * NRF; t += nth) {
-        int c = t / (NGF * NRF), gf = (t / NRF) % NGF, beta = t % NRF;
-        const double* P = ptf + (f * NGF + gf) * C::PT_FACE;
-        const double* U0 = P + M;
-        const double* U1 = U0 + M * M;
-        const double* U2 = U1 + M * M;
-        double psi = T.PhiF[(f * NGF + gf) * NP + T.fnodes[f * NFN + c]];
-        double u;
-        if (beta == 0)
-          u = U0[i * M + l];
-        else if (beta == 1)
-          u = U1[i * M + l];
-        else
-          u = U2[(i * M + l) * D + (beta - 2)];
-        Zs[t] = psi * u;
-      }
-      __syncthreads();
-      for (int t = tid; t < NFN * NZ; t += nth) {
-        int c = t / NZ, j = t % NZ;
-        double acc = 0.0;
-        for (int gf = 0; gf < NGF; ++gf)
-          for (int beta = 0; beta < NRF; ++beta) acc += Zs[(c * NGF + gf) * NRF + beta] * Rb[(beta * NGF + gf) * NZ + j];
-        int rowv = T.fnodes[f * NFN + c] * M + i;
-        int rowt = (f * NFN + c) * M + i;
-        if (j < NP) {
-          Ap[rowv * NV + j * M + l] += acc;
-          Cp[rowt * NV + j * M + l] = acc;
-        } else {
-          int tcol = (j - NP) * M + l;
-          Bp[rowv * NT + tcol] += acc;
-          Dp[rowt * NT + tcol] = acc;
-        }
-      }
-    }
-  }
-  __syncthreads();
-  double* Rout = a.R + e * (int64_t)(NV + NT);
-  for (int t = tid; t < NV; t += nth) Rout[t] = Rv[t];
-  for (int t = tid; t < NT; t += nth) Rout[NV + t] = Rt[t];
+  double* R = a.R + e * (int64_t)(NV + NT);
+  const UniformDims<C> d;
+  element_residual<D, NTH>(d, E, ptv, ptf, a.hist ? a.hist + e * NV : nullptr, R, R + NV);
+  element_blocks<D, C::VISC, NTH, AsmSmem<C>::NRD>(d, E, ptv, ptf, a.Ap + le * NV * NV,
+                                                   a.recov + e * (int64_t)(NV * NT + NV), a.Cp + le * NT * NV,
+                                                   a.S + e * (int64_t)NT * NT, smem);
 }
 
 // ------------------------------------------------------------------------------------
-// k_condense
+// k_condense: one CTA per element, LU in shared memory (two CTAs per SM at 3D p = 3)
 // ------------------------------------------------------------------------------------
 template <class C>
 struct CondSmem {
-  static constexpr int CB = 64;  // right-hand-side columns per block
-  static constexpr size_t bytes = sizeof(double) * (C::NV * C::NV + C::NV * CB) + sizeof(int) * C::NV + 64;
+  static constexpr int NTH = C::NV <= 24 ? 64 : C::NV <= 64 ? 128 : 256;
+  // right-hand-side columns per block: all of them, or 40 (a divisor of 3D's 120 and 200; the most that
+  // lets two CTAs share an SM at p = 3)
+  static constexpr int CB = C::NT <= 60 ? (C::NT + 3) / 4 * 4 : 40;
+  static constexpr int LD = C::NV % 2 ? C::NV + 2 : C::NV + 1;  // odd (a column's entries lie in different banks), > NV
+  static constexpr int LUN = (C::NV * LD + 1) / 2 * 2;
+  static constexpr size_t bytes = sizeof(double) * (LUN + C::NV * CB + 2 * C::NV) + sizeof(int) * C::NV;
 };
 
 template <class C>
-__global__ void __launch_bounds__(256) k_condense(AssembleArgs a) {
+__global__ void __launch_bounds__(CondSmem<C>::NTH, 512 / CondSmem<C>::NTH) k_condense(AssembleArgs a) {
   constexpr int NV = C::NV, NT = C::NT;
   using SM = CondSmem<C>;
-  constexpr int CB = SM::CB;
-  extern __shared__ double smem[];
-  double* LU = smem;                 // [NV][NV]
-  double* Xs = LU + NV * NV;         // [NV][CB]
-  int* piv = reinterpret_cast<int*>(Xs + NV * CB);
-  __shared__ int s_piv;
-  __shared__ int s_bad;
+  extern __shared__ __align__(16) double smem[];
+  double* LU = smem;                 // [NV][LD]: A' and R_v
+  double* Xs = LU + SM::LUN;         // [NV][CB]
+  double* dinv = Xs + NV * SM::CB;   // [NV]
+  double* ys = dinv + NV;            // [NV]
+  int* perm = reinterpret_cast<int*>(ys + NV);
+  __shared__ int s_piv[2];
   const int64_t le = blockIdx.x;
   const int64_t e = a.e0 + le;
   if (skip_element(a, e)) return;
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = threadIdx.x;
   const double* Ap = a.Ap + le * NV * NV;
-  const double* Cp = a.Cp + le * NT * NV;
-  double* X = a.recov + e * (int64_t)(NV * NT + NV);
-  double* y = X + NV * NT;
-  double* S = a.S + e * (int64_t)NT * NT;
   const double* R = a.R + e * (int64_t)(NV + NT);
-  for (int t = tid; t < NV * NV; t += nth) LU[t] = Ap[t];
-  if (tid == 0) s_bad = 0;
+  double* X = a.recov + e * (int64_t)(NV * NT + NV);
+  for (int t = tid; t < NV * NV; t += SM::NTH) LU[t / NV * SM::LD + t % NV] = Ap[t];
+  for (int t = tid; t < NV; t += SM::NTH) LU[t * SM::LD + NV] = R[t];
   __syncthreads();
-  // LU with partial pivoting (row interchanges recorded in piv)
-  for (int k = 0; k < NV; ++k) {
-    if (tid < 32) {
-      double best = -1.0;
-      int bi = k;
-      for (int r = k + tid; r < NV; r += 32) {
-        double v = fabs(LU[r * NV + k]);
-        if (v > best) {
-          best = v;
-          bi = r;
-        }
-      }
-      for (int off = 16; off > 0; off >>= 1) {
-        double ob = __shfl_down_sync(0xffffffffu, best, off);
-        int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      if (tid == 0) {
-        s_piv = bi;
-        piv[k] = bi;
-        if (!(best > 0.0)) s_bad = 1;
-      }
-    }
-    __syncthreads();
-    const int pr = s_piv;
-    if (pr != k)
-      for (int j = tid; j < NV; j += nth) {
-        double t = LU[k * NV + j];
-        LU[k * NV + j] = LU[pr * NV + j];
-        LU[pr * NV + j] = t;
-      }
-    __syncthreads();
-    const double d = LU[k * NV + k];
-    const double inv = d != 0.0 ? 1.0 / d : 0.0;
-    for (int r = k + 1 + tid; r < NV; r += nth) LU[r * NV + k] *= inv;
-    __syncthreads();
-    const int rem = NV - k - 1;
-    for (int t = tid; t < rem * rem; t += nth) {
-      int r = k + 1 + t / rem, c = k + 1 + t % rem;
-      LU[r * NV + c] -= LU[r * NV + k] * LU[k * NV + c];
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && s_bad) atomicOr(a.status + e, HDG_STATUS_SINGULAR);
-  // X = A'^{-1} [B' | R_v] in column blocks (B' stored in X)
-  for (int c0 = 0; c0 < NT + 1; c0 += CB) {
-    const int nc = (NT + 1 - c0) < CB ? (NT + 1 - c0) : CB;
-    __syncthreads();
-    for (int t = tid; t < NV * CB; t += nth) {
-      int r = t / CB, c = t % CB;
-      int col = c0 + c;
-      double v = 0.0;
-      if (c < nc) v = col < NT ? X[r * NT + col] : R[r];
-      Xs[t] = v;
-    }
-    __syncthreads();
-    // apply the row interchanges in order
-    for (int t = tid; t < CB; t += nth)
-      for (int k = 0; k < NV; ++k) {
-        int p = piv[k];
-        if (p != k) {
-          double tmp = Xs[k * CB + t];
-          Xs[k * CB + t] = Xs[p * CB + t];
-          Xs[p * CB + t] = tmp;
-        }
-      }
-    __syncthreads();
-    for (int k = 0; k < NV; ++k) {  // forward, unit lower
-      for (int t = tid; t < (NV - k - 1) * CB; t += nth) {
-        int r = k + 1 + t / CB, c = t % CB;
-        Xs[r * CB + c] -= LU[r * NV + k] * Xs[k * CB + c];
-      }
-      __syncthreads();
-    }
-    for (int k = NV - 1; k >= 0; --k) {  // backward, upper
-      for (int c = tid; c < CB; c += nth) Xs[k * CB + c] /= LU[k * NV + k];
-      __syncthreads();
-      for (int t = tid; t < k * CB; t += nth) {
-        int r = t / CB, c = t % CB;
-        Xs[r * CB + c] -= LU[r * NV + k] * Xs[k * CB + c];
-      }
-      __syncthreads();
-    }
-    for (int t = tid; t < NV * CB; t += nth) {
-      int r = t / CB, c = t % CB;
-      int col = c0 + c;
-      if (c < nc) {
-        if (col < NT)
-          X[r * NT + col] = Xs[t];
-        else
-          y[r] = Xs[t];
-      }
-    }
-  }
-  __syncthreads();
-  // S = D' - C' X ; g = R_t - C' y
-  for (int t = tid; t < NT * NT; t += nth) {
-    int r = t / NT, c = t % NT;
-    double s = S[t];
-    const double* Cr = Cp + r * NV;
-    for (int k = 0; k < NV; ++k) s -= Cr[k] * X[k * NT + c];
-    S[t] = s;
-  }
-  double* g = a.g + e * NT;
-  for (int r = tid; r < NT; r += nth) {
-    double s = R[NV + r];
-    const double* Cr = Cp + r * NV;
-    for (int k = 0; k < NV; ++k) s -= Cr[k] * y[k];
-    g[r] = s;
-  }
+  const bool ok = element_condense<SM::NTH, SM::CB>(LU, SM::LD, NV, perm, dinv, ys, s_piv, Xs, a.Cp + le * NT * NV,
+                                                    R + NV, X, X + NV * NT, a.S + e * (int64_t)NT * NT,
+                                                    a.g + e * NT, NT);
+  if (tid == 0 && !ok) atomicOr(a.status + e, HDG_STATUS_SINGULAR);
   if (a.only_flag != 0 && tid == 0) {  // flagged-only pass: the block is now the FP64 form's
     atomicAnd(a.status + e, ~a.only_flag);
     atomicOr(a.status + e, HDG_STATUS_FP64);

@@ -311,12 +311,12 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
       }
       {
         LaunchScope ls(ctx, HDG_KERNEL_ASSEMBLE, s);
-        k_assemble<C><<<(unsigned)a.ne, 256, AsmSmem<C>::bytes, s>>>(f, ctx->T);
+        k_assemble<C><<<(unsigned)a.ne, AsmSmem<C>::NTH, AsmSmem<C>::bytes, s>>>(f, ctx->T);
       }
       if (int rc_b = boundary_patch(ctx, f, HDG_PREC_FP64, s)) return rc_b;
       {
         LaunchScope ls(ctx, HDG_KERNEL_CONDENSE, s);
-        k_condense<C><<<(unsigned)a.ne, 256, CondSmem<C>::bytes, s>>>(f);
+        k_condense<C><<<(unsigned)a.ne, CondSmem<C>::NTH, CondSmem<C>::bytes, s>>>(f);
       }
     }
     if (int rc_d = chunk_done(ctx, e0, a.ne, s)) return rc_d;

@@ -400,9 +400,10 @@ int hdg_ctx_create(hdg_mesh_t mesh, const hdg_physics* phys, int device, hdg_ctx
 
   hdg::RefTables T = hdg::make_tables(m.ref);
   std::vector<double> tab;
-  size_t off[8];
-  const std::vector<double>* parts[8] = {&T.W, &T.Phi, &T.dPhi, &T.PL, &T.WF, &T.PhiF, &T.dPhiF, &T.PLF};
-  for (int i = 0; i < 8; ++i) {
+  size_t off[11];
+  const std::vector<double>* parts[11] = {&T.W,     &T.Phi, &T.dPhi, &T.PL,  &T.WF, &T.PhiF,
+                                          &T.dPhiF, &T.PLF, &T.dR,   &T.dRF, &T.Psi};
+  for (int i = 0; i < 11; ++i) {
     off[i] = tab.size();
     tab.insert(tab.end(), parts[i]->begin(), parts[i]->end());
   }
@@ -496,6 +497,9 @@ int hdg_ctx_create(hdg_mesh_t mesh, const hdg_physics* phys, int device, hdg_ctx
   c->T.PhiF = c->d_tab + off[5];
   c->T.dPhiF = c->d_tab + off[6];
   c->T.PLF = c->d_tab + off[7];
+  c->T.dR = c->d_tab + off[8];
+  c->T.dRF = c->d_tab + off[9];
+  c->T.Psi = c->d_tab + off[10];
   c->T.fnodes = c->d_itab;
   c->T.nodepos = c->d_itab + npos_off;
   *out = c;

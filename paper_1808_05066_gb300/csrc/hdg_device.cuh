@@ -57,6 +57,9 @@ struct DevTables {
   const double* PhiF;   // [NF][NGF][NP]
   const double* dPhiF;  // [NF][D][NGF][NP]
   const double* PLF;    // [NF][NF][NGF][NFN]
+  const double* dR;     // [D][NG][NP]       lifted-gradient operators in reference coordinates
+  const double* dRF;    // [NF][D][NGF][NP]
+  const double* Psi;    // [NF][NGF][NFN]    the face's own basis functions at its points
   const int* fnodes;    // [NF][NFN]
   const int* nodepos;   // [NF][NP] position of node a on face f, -1 if off the face
 };
@@ -425,6 +428,38 @@ HDG_DEVI void visc_jac_dir(const ViscFactors<D>& f, const double* c, const PhysP
     }
     emit(M - 1, M - 1, k, -ph.mu * (VA * c[k] + f.vel[k] * cA - t3 * f.A[k] * cV) - kc * c[k]);
   }
+}
+
+// sum_jk c_j c2_k dG_ij/dq_lk: visc_jac_dir contracted with a second vector, for i, l >= 1 (the
+// other entries vanish). emit(i, l, value).
+template <int D, class Emit>
+HDG_DEVI void visc_jac_pair(const ViscFactors<D>& f, const double* c, const double* c2, const PhysParams& ph,
+                            Emit emit) {
+  constexpr int M = D + 2;
+  constexpr double t3 = 2.0 / 3.0;
+  double cc = 0.0, cA = 0.0, cV = 0.0, eA = 0.0, eV = 0.0, VA = 0.0;
+#pragma unroll
+  for (int j = 0; j < D; ++j) {
+    cc += c[j] * c2[j];
+    cA += c[j] * f.A[j];
+    cV += c[j] * f.vel[j];
+    eA += c2[j] * f.A[j];
+    eV += c2[j] * f.vel[j];
+    VA += f.vel[j] * f.A[j];
+  }
+  const double mi = ph.mu * f.ivm, kc = (ph.kappa / ph.cv) * f.ivm2;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+#pragma unroll
+    for (int b = 0; b < D; ++b) {
+      double s = c2[a] * c[b] - t3 * (c[a] * c2[b]);
+      if (a == b) s += cc;
+      emit(1 + a, 1 + b, mi * s);
+    }
+    emit(1 + a, M - 1, -ph.mu * (f.A[a] * cc + c2[a] * cA - t3 * (eA * c[a])));
+    emit(M - 1, 1 + a, mi * (f.vel[a] * cc + eV * c[a] - t3 * (c2[a] * cV)));
+  }
+  emit(M - 1, M - 1, -ph.mu * (VA * cc + eV * cA - t3 * (eA * cV)) - kc * cc);
 }
 
 // Largest-magnitude eigenvalue of A_n: |V.n| + c (Eq. sLxF).

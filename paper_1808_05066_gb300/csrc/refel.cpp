@@ -291,6 +291,28 @@ RefTables make_tables(const RefElement& r) {
           for (int b = 0; b < Np; ++b) s += T.PhiF[(f * NGF + g) * Np + b] * L[(fl * Np + b) * Nf + c];
           T.PLF[((f * nF + fl) * NGF + g) * Nf + c] = s;
         }
+  // reference lifted gradients of the element functions, and the faces' own basis functions
+  auto lift_at = [&](const double* pl, int f, int a) {  // pl: lift values of face f's functions at a point
+    for (int c = 0; c < Nf; ++c)
+      if (r.face_nodes[f][c] == a) return pl[c];
+    return 0.0;
+  };
+  T.dR = T.dPhi;
+  for (int s = 0; s < d; ++s)
+    for (int g = 0; g < NG; ++g)
+      for (int a = 0; a < Np; ++a)
+        T.dR[(s * NG + g) * Np + a] +=
+            lift_at(&T.PL[((s + 1) * NG + g) * Nf], s + 1, a) - lift_at(&T.PL[g * Nf], 0, a);
+  T.dRF = T.dPhiF;
+  T.Psi.resize(nF * NGF * Nf);
+  for (int f = 0; f < nF; ++f)
+    for (int g = 0; g < NGF; ++g) {
+      for (int s = 0; s < d; ++s)
+        for (int a = 0; a < Np; ++a)
+          T.dRF[((f * d + s) * NGF + g) * Np + a] += lift_at(&T.PLF[((f * nF + s + 1) * NGF + g) * Nf], s + 1, a) -
+                                                     lift_at(&T.PLF[(f * nF * NGF + g) * Nf], 0, a);
+      for (int c = 0; c < Nf; ++c) T.Psi[(f * NGF + g) * Nf + c] = T.PhiF[(f * NGF + g) * Np + r.face_nodes[f][c]];
+    }
   return T;
 }
 

@@ -50,6 +50,11 @@ struct RefTables {
   std::vector<double> PhiF;   // [nF][NGF][Np]   element basis at face-f points
   std::vector<double> dPhiF;  // [nF][dim][NGF][Np]
   std::vector<double> PLF;    // [nF(face pts)][nF(lift)][NGF][Nf]
+  // the lifted gradient of element function j in reference coordinates, with n_f |F| / |K| written as
+  // -Jinv row f - 1 (f > 0) or the sum of the rows (f = 0): dPhi_r + PL_{r+1} phi_j - PL_0 phi_j
+  std::vector<double> dR;     // [dim][NG][Np]
+  std::vector<double> dRF;    // [nF][dim][NGF][Np]
+  std::vector<double> Psi;    // [nF][NGF][Nf]   element basis of face f's nodes at its points
   std::vector<double> Mref;   // [Np][Np] reference mass matrix
   std::vector<int> fnodes;    // [nF][Nf] element node of face node c
 };
