@@ -412,8 +412,7 @@ struct AsmSmem {
   static constexpr int TILES = UniformDims<C>::NPs / 2 * (UniformDims<C>::NPs / 2 + (C::VISC ? (C::NFN + 1) / 2 : 0));
   static constexpr int NRD = (TILES + NTH - 1) / NTH;
   static constexpr int MINB = NTH == 256 ? 3 : 5;  // registers: 80 a thread
-  static constexpr int H = C::NF * C::NGF * UniformDims<C>::NZs, Z = 2 * C::NG * UniformDims<C>::NPs;
-  static constexpr size_t bytes = sizeof(double) * (UniformDims<C>::NTN * UniformDims<C>::NZs + (H > Z ? H : Z));
+  static constexpr size_t bytes = sizeof(double) * element_smem_doubles(UniformDims<C>(), C::NF, 2);
 };
 
 // the reference operators of an element of one degree, filled in by one thread
@@ -455,7 +454,7 @@ __global__ void __launch_bounds__(AsmSmem<C>::NTH, AsmSmem<C>::MINB) k_assemble(
   double* R = a.R + e * (int64_t)(NV + NT);
   const UniformDims<C> d;
   element_residual<D, NTH>(d, E, ptv, ptf, a.hist ? a.hist + e * NV : nullptr, R, R + NV);
-  element_blocks<D, C::VISC, NTH, AsmSmem<C>::NRD>(d, E, ptv, ptf, a.Ap + le * NV * NV,
+  element_blocks<D, C::VISC, NTH, AsmSmem<C>::NRD, NF, 2>(d, E, ptv, ptf, a.Ap + le * NV * NV,
                                                    a.recov + e * (int64_t)(NV * NT + NV), a.Cp + le * NT * NV,
                                                    a.S + e * (int64_t)NT * NT, smem);
 }

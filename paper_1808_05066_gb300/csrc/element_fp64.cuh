@@ -39,9 +39,10 @@ struct ElemTables {
 
 // Sizes of the contraction: any type with members NP, NG, NGF, NTN (trace nodes), NPs, NZs (NP and
 // NP + trace nodes with every group padded to an even count) and NV, NT.
+// FB faces share one pass over the trial side, ZB left factors are buffered.
 template <class Dm>
-HDG_DEVI constexpr int element_smem_doubles(const Dm& d, int nf) {
-  const int h = nf * d.NGF * d.NZs, z = 2 * d.NG * d.NPs;
+__host__ __device__ constexpr int element_smem_doubles(const Dm& d, int FB, int ZB) {
+  const int h = FB * d.NGF * d.NZs, z = ZB * d.NG * d.NPs;
   return d.NTN * d.NZs + (h > z ? h : z);
 }
 
@@ -88,8 +89,9 @@ HDG_DEVI void element_residual(const Dm& d, const ElemTables<D>& T, const double
 // shared buffers while the other one is multiplied. One operator's 2 x 2 tiles, those of A' and
 // then those of one face's block of B', are one list over the threads (NRD rounds), so that only
 // the list's last warp is partly filled; A' tiles stay in registers over the operators, a trace
-// face's block is complete after one.
-template <int D, bool VISC, int NTH, int NRD, class Dm>
+// face's block is complete after one. Large classes take one face per pass and one left factor
+// (FB = ZB = 1), so that two CTAs still share an SM.
+template <int D, bool VISC, int NTH, int NRD, int FB, int ZB, class Dm>
 HDG_DEVI void element_blocks(const Dm& d, const ElemTables<D>& T, const double* __restrict__ ptv,
                              const double* __restrict__ ptf, double* Ap, double* Bp, double* Cp, double* Dp,
                              double* sm) {
@@ -97,8 +99,8 @@ HDG_DEVI void element_blocks(const Dm& d, const ElemTables<D>& T, const double* 
   const int NP = d.NP, NG = d.NG, NGF = d.NGF, NTN = d.NTN, NPs = d.NPs, NZs = d.NZs, NV = d.NV, NT = d.NT;
   const int NQ = NF * NGF, tid = threadIdx.x;
   double* F = sm;               // [NTN][NZs]
-  double* H = F + NTN * NZs;    // [NQ][NZs]
-  double* Z = H;                // [2][NG][NPs], after H
+  double* H = F + NTN * NZs;    // [FB NGF][NZs]
+  double* Z = H;                // [ZB][NG][NPs], after H
   const double* T0 = ptv + (M + D * M) * NG;
   const double* T1 = T0 + M * M * NG;
   const double* T2 = T1 + D * M * M * NG;
@@ -111,92 +113,94 @@ HDG_DEVI void element_blocks(const Dm& d, const ElemTables<D>& T, const double* 
     const int i = il / M, l = il % M;
     const bool visc = VISC && i > 0 && l > 0;
     const int iv = visc ? (i - 1) * MV + (l - 1) : 0;
-    // trial side of the faces
-    for (int t = tid; t < NQ * NZs; t += NTH) {
-      const int p = t / NZs, col = t % NZs, f = p / NGF, gf = p % NGF;
-      double v = 0.0;
-      if (col < NPs) {
-        if (col < NP) {
-          v = U0[il * NQ + p] * T.PhiF[p * NP + col];
-          if (visc)
+    for (int f0 = 0; f0 < NF; f0 += FB) {
+      // trial side of FB faces
+      for (int t = tid; t < FB * NGF * NZs; t += NTH) {
+        const int p = f0 * NGF + t / NZs, col = t % NZs, f = p / NGF, gf = p % NGF;
+        double v = 0.0;
+        if (col < NPs) {
+          if (col < NP) {
+            v = U0[il * NQ + p] * T.PhiF[p * NP + col];
+            if (visc)
 #pragma unroll
-            for (int r = 0; r < D; ++r)
-              v += U2[(r * MV * MV + iv) * NQ + p] * T.dRF[((f * D + r) * NGF + gf) * NP + col];
-        }
-      } else {
-        const int tp = col - NPs;
-        int fl = 0;
-        while (tp >= T.offp[fl + 1]) ++fl;
-        const int c = tp - T.offp[fl], nq = T.nq[fl];
-        if (c < nq) {
-          if (fl == f) v = U1[il * NQ + p] * T.Psi[f][gf * nq + c];
-          if (visc) {
-            const double u = fl > 0 ? -U2[((fl - 1) * MV * MV + iv) * NQ + p] : U2[(D * MV * MV + iv) * NQ + p];
-            v += u * T.PLF[fl][f * T.sPLF[fl] + gf * nq + c];
+              for (int r = 0; r < D; ++r)
+                v += U2[(r * MV * MV + iv) * NQ + p] * T.dRF[((f * D + r) * NGF + gf) * NP + col];
+          }
+        } else {
+          const int tp = col - NPs;
+          int fl = 0;
+          while (tp >= T.offp[fl + 1]) ++fl;
+          const int c = tp - T.offp[fl], nq = T.nq[fl];
+          if (c < nq) {
+            if (fl == f) v = U1[il * NQ + p] * T.Psi[f][gf * nq + c];
+            if (visc) {
+              const double u = fl > 0 ? -U2[((fl - 1) * MV * MV + iv) * NQ + p] : U2[(D * MV * MV + iv) * NQ + p];
+              v += u * T.PLF[fl][f * T.sPLF[fl] + gf * nq + c];
+            }
           }
         }
+        H[t] = v;
       }
-      H[t] = v;
-    }
-    __syncthreads();
-    // face rows: 2 x 2 tiles; a pair without the viscous part reaches the face's own trace columns only
-    {
-      int nqm = 0;
+      __syncthreads();
+      // face rows: 2 x 2 tiles; a pair without the viscous part reaches the face's own trace columns only
+      {
+        int nqm = 0;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) nqm = max(nqm, T.offp[f + 1] - T.offp[f]);
-      const int ncp = visc ? NZs / 2 : (NPs + nqm) / 2, nrp = T.offp[NF] / 2;
-      for (int t = tid; t < nrp * ncp; t += NTH) {
-        const int rp = t / ncp, cp = t % ncp;
-        int f = 0;
-        while (2 * rp >= T.offp[f + 1]) ++f;
-        const int c0 = 2 * rp - T.offp[f], nq = T.nq[f];
-        int col = 2 * cp, fl = -1, cc = col;  // fl: face of the trace columns, cc: column within the group
-        if (col >= NPs) {
-          if (visc) {
-            fl = 0;
-            while (col - NPs >= T.offp[fl + 1]) ++fl;
-            cc = col - NPs - T.offp[fl];
-          } else {
-            fl = f;
-            cc = col - NPs;
-            col = NPs + T.offp[f] + cc;
-          }
-          if (cc >= T.nq[fl]) continue;
-        }
-        const bool r1 = c0 + 1 < nq;
-        const double* psi = T.Psi[f] + c0;
-        const double* h = H + f * NGF * NZs + col;
-        double a00 = 0.0, a01 = 0.0, a10 = 0.0, a11 = 0.0;
-#pragma unroll 4
-        for (int gf = 0; gf < NGF; ++gf) {
-          const double p0 = psi[gf * nq], p1 = r1 ? psi[gf * nq + 1] : 0.0;
-          const double2 hv = *reinterpret_cast<const double2*>(h + gf * NZs);
-          a00 += p0 * hv.x;
-          a01 += p0 * hv.y;
-          a10 += p1 * hv.x;
-          a11 += p1 * hv.y;
-        }
-        const bool k1 = cc + 1 < (fl < 0 ? NP : T.nq[fl]);
-#pragma unroll
-        for (int rr = 0; rr < 2; ++rr) {
-          if (rr && !r1) break;
-          const int tn = T.off[f] + c0 + rr, row = tn * M + i;
-          const double v0 = rr ? a10 : a00, v1 = rr ? a11 : a01;
-          *reinterpret_cast<double2*>(F + tn * NZs + col) = make_double2(v0, v1);
-          double* dst = fl < 0 ? Cp + (int64_t)row * NV + cc * M + l : Dp + (int64_t)row * NT + (T.off[fl] + cc) * M + l;
-          dst[0] = v0;
-          if (k1) dst[M] = v1;
-        }
-      }
-      if (!visc)  // the other faces' columns of D' are zero for this pair
-        for (int t = tid; t < NTN * NTN; t += NTH) {
-          const int r = t / NTN, c = t % NTN;
+        for (int f = 0; f < NF; ++f) nqm = max(nqm, T.offp[f + 1] - T.offp[f]);
+        const int ncp = visc ? NZs / 2 : (NPs + nqm) / 2, rp0 = T.offp[f0] / 2, nrp = T.offp[f0 + FB] / 2 - rp0;
+        for (int t = tid; t < nrp * ncp; t += NTH) {
+          const int rp = rp0 + t / ncp, cp = t % ncp;
           int f = 0;
-          while (r >= T.off[f + 1]) ++f;
-          if (c < T.off[f] || c >= T.off[f + 1]) Dp[(int64_t)(r * M + i) * NT + c * M + l] = 0.0;
+          while (2 * rp >= T.offp[f + 1]) ++f;
+          const int c0 = 2 * rp - T.offp[f], nq = T.nq[f];
+          int col = 2 * cp, fl = -1, cc = col;  // fl: face of the trace columns, cc: column within the group
+          if (col >= NPs) {
+            if (visc) {
+              fl = 0;
+              while (col - NPs >= T.offp[fl + 1]) ++fl;
+              cc = col - NPs - T.offp[fl];
+            } else {
+              fl = f;
+              cc = col - NPs;
+              col = NPs + T.offp[f] + cc;
+            }
+            if (cc >= T.nq[fl]) continue;
+          }
+          const bool r1 = c0 + 1 < nq;
+          const double* psi = T.Psi[f] + c0;
+          const double* h = H + (f - f0) * NGF * NZs + col;
+          double a00 = 0.0, a01 = 0.0, a10 = 0.0, a11 = 0.0;
+#pragma unroll 4
+          for (int gf = 0; gf < NGF; ++gf) {
+            const double p0 = psi[gf * nq], p1 = r1 ? psi[gf * nq + 1] : 0.0;
+            const double2 hv = *reinterpret_cast<const double2*>(h + gf * NZs);
+            a00 += p0 * hv.x;
+            a01 += p0 * hv.y;
+            a10 += p1 * hv.x;
+            a11 += p1 * hv.y;
+          }
+          const bool k1 = cc + 1 < (fl < 0 ? NP : T.nq[fl]);
+#pragma unroll
+          for (int rr = 0; rr < 2; ++rr) {
+            if (rr && !r1) break;
+            const int tn = T.off[f] + c0 + rr, row = tn * M + i;
+            const double v0 = rr ? a10 : a00, v1 = rr ? a11 : a01;
+            *reinterpret_cast<double2*>(F + tn * NZs + col) = make_double2(v0, v1);
+            double* dst = fl < 0 ? Cp + (int64_t)row * NV + cc * M + l : Dp + (int64_t)row * NT + (T.off[fl] + cc) * M + l;
+            dst[0] = v0;
+            if (k1) dst[M] = v1;
+          }
         }
+        if (!visc && f0 == 0)  // the other faces' columns of D' are zero for this pair
+          for (int t = tid; t < NTN * NTN; t += NTH) {
+            const int r = t / NTN, c = t % NTN;
+            int f = 0;
+            while (r >= T.off[f + 1]) ++f;
+            if (c < T.off[f] || c >= T.off[f + 1]) Dp[(int64_t)(r * M + i) * NT + c * M + l] = 0.0;
+          }
+      }
+      __syncthreads();
     }
-    __syncthreads();
     // F's share of entry (test node a, column position col of F)
     auto face_part = [&](int a, int col, int f) {
       const int pos = T.nodepos[f * NP + a];
@@ -231,8 +235,8 @@ HDG_DEVI void element_blocks(const Dm& d, const ElemTables<D>& T, const double* 
     build(0, Z);
     __syncthreads();
     for (int o = 0; o < nops; ++o) {
-      const double* Zb = Z + (o & 1) * NG * NPs;
-      if (o + 1 < nops) build(o + 1, Z + ((o + 1) & 1) * NG * NPs);
+      const double* Zb = Z + (o % ZB) * NG * NPs;
+      if (ZB > 1 && o + 1 < nops) build(o + 1, Z + ((o + 1) % ZB) * NG * NPs);
       const int f = o <= D ? o : 0;  // the face of this operator's trace columns (o >= 1)
       const int nA = o <= D ? nAt : 0, tq = o >= 1 ? (T.nq[f] + 1) / 2 : 0, n = nAt + tA * tq;
 #pragma unroll
@@ -268,6 +272,10 @@ HDG_DEVI void element_blocks(const Dm& d, const ElemTables<D>& T, const double* 
         }
       }
       __syncthreads();
+      if (ZB == 1 && o + 1 < nops) {
+        build(o + 1, Z);
+        __syncthreads();
+      }
     }
 #pragma unroll
     for (int x = 0; x < NRD; ++x) {
@@ -391,7 +399,7 @@ template <int NTH, int CB>
 HDG_DEVI void element_solve_schur(const double* LU, int ld, int n, const int* perm, const double* dinv, double* Xs,
                                   const double* Cp, double* X, double* S, int nt) {
   constexpr int NB = 8;
-  static_assert(CB % 4 == 0 && CB <= NTH, "tiles");
+  static_assert(CB % 4 == 0 && CB <= NTH && NTH % 32 == 0, "tiles");
   const int tid = threadIdx.x;
   for (int c0 = 0; c0 < nt; c0 += CB) {
     const int nc = min(CB, nt - c0), nct = (nc + 3) / 4;

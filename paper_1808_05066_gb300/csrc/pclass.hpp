@@ -13,17 +13,20 @@ namespace hdg {
 
 constexpr int kPClasses = 10;  // (pk, pt) with 1 <= pk <= pt <= 4 (3D Navier-Stokes)
 
-// sizes of one (pk, pt) class: nodes, points, unknowns, tiles, shared memory and per-CTA scratch
-// (doubles) of the fused kernel
+// sizes of one (pk, pt) class: nodes, points, unknowns, shared memory and per-CTA scratch (doubles) of
+// the fused kernel
 struct PDims {
-  int pk, pt, NP, NFK, NFN, NG, NGF, NV, NT, NZ, GT, CB, RBMAX, ASM, CND, KEEP, SMEM, lu_smem;
+  int pk, pt, NP, NFK, NFN, NG, NGF, NV, NT, NZ, SMEM;
   int64_t SLOT;
 };
 
-// device pointers of the tables of one (pk, pt) class (layouts of ClassTables, refel.hpp) and its sizes
+// device pointers of the tables of one (pk, pt) class and its sizes (layouts of ClassTables, refel.hpp;
+// dR, dRF and the tables of a face's own trace degree q in element_fp64.cuh's layouts, every face)
 struct PClassDev {
-  const double *W, *Phi, *dPhi, *WF, *PhiF, *dPhiF, *PsiF, *PhiN, *PL, *PLF, *PLV, *PLFV, *IPro;
-  const int* fnodesK;
+  const double *W, *Phi, *dPhi, *dR, *WF, *PhiF, *dPhiF, *dRF, *PsiF, *PhiN, *PL, *PLF, *IPro;
+  const double *PsiQ[4], *PLQ[4], *PLFQ[4], *TrQ[4];  // [q - 1]: [NF][NGF][nq], [NF][NG][nq], [NF][NF][NGF][nq],
+                                                      // [NF][nq][NP]; q <= pt (TrQ: pk <= q)
+  const int* nodepos;                                 // [NF][NP]
   PDims d;
 };
 
@@ -50,10 +53,7 @@ struct PMix {
   PClassDev tab[kPClasses] = {};
   int64_t class_count[kPClasses] = {};
   size_t smem_bytes = 0;      // dynamic shared memory of the launch: the largest class present
-  size_t smem_limit = 0;      // dynamic shared memory a CTA of the fused kernel may use on the device
-  bool tuned = false;         // tile shapes (GT, CB) chosen per class by timing (first call)
-  std::vector<int> h_queue;   // host copy of the queue
-  std::vector<int8_t> h_cls;  // host copy of the classes
+  int ctas = 0;               // CTAs of the persistent launch
   int64_t slot_doubles = 0;   // per-CTA scratch: the largest class present
   bool attr_set = false;
 };
