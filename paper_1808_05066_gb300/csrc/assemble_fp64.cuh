@@ -21,8 +21,6 @@
 //   k_condense   one CTA per element: LU with partial pivoting of A' in shared memory,
 //                triangular solves for X and y, Schur products for S and g.
 #pragma once
-#include <type_traits>
-
 #include "dfloat.cuh"
 #include "element_fp64.cuh"
 #include "hdg_device.cuh"
@@ -44,7 +42,6 @@ struct AssembleArgs {
   double* Cp;           // [ne][NT][NV]
   uint4* oz;            // [ne][...] exact-slice operands of the mixed condensation
   float* prep;          // [ne][...] inverse, FP32 copy and scales for the mixed condensation
-  uint2* rb;            // [ne][...] operator slices of the mixed assembly
   // outputs (global element index)
   double* S;            // [E][NT][NT]   (D' on entry to condense)
   double* g;            // [E][NT]
@@ -125,17 +122,16 @@ HDG_DEVI void volume_point_state(int g, const DevTables& T, const double (*z)[C:
 HDG_DEVI void put(double* p, int i, double v) { p[i] = v; }
 HDG_DEVI void put(df2* p, int i, double v) { p[i] = df_from(v); }
 
-// Point tensors of one point: the FP64 form stores them [quantity][point] (element_fp64.cuh: the
-// contractions read one quantity over the points), the mixed form [point][quantity].
-template <class OutT, int NPT>
+// Point tensors are stored [quantity][point] (element_fp64.cuh: the contractions read one quantity over
+// the points); PtOut addresses those of one point.
+template <int NPT>
 struct PtOut {
-  static constexpr int S = std::is_same<OutT, double>::value ? NPT : 1;
-  OutT* p;
-  HDG_DEVI PtOut operator+(int i) const { return {p + i * S}; }
+  double* p;
+  HDG_DEVI PtOut operator+(int i) const { return {p + i * NPT}; }
 };
-template <class OutT, int NPT>
-HDG_DEVI void put(const PtOut<OutT, NPT>& o, int i, double v) {
-  put(o.p, i * PtOut<OutT, NPT>::S, v);
+template <int NPT>
+HDG_DEVI void put(const PtOut<NPT>& o, int i, double v) {
+  o.p[i * NPT] = v;
 }
 
 // row r of Jinv, or the sum of the rows (r = D)
@@ -165,9 +161,8 @@ struct SigmaValues<M, true> {
   HDG_DEVI double operator()(int i, int l) const { return s[i][l]; }
 };
 
-// OutT = double (FP64 form) or df2 (mixed form: per-point tensors as double-floats);
 // SYM: sigma_S of Eq. symStab instead of sigma_SLF (launch through launch_pointwise).
-template <class C, class OutT = double, bool SYM = false>
+template <class C, bool SYM = false>
 __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, PhysParams ph) {
   constexpr int D = C::D, M = C::M, NP = C::NP, NFN = C::NFN, NF = C::NF, NG = C::NG, NGF = C::NGF;
   __shared__ double z[C::NZ][M];
@@ -210,8 +205,8 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
       for (int i = 0; i < M; ++i)
         for (int j = 0; j < D; ++j) F[i][j] = F[i][j] + Gv[i][j];
     }
-    using Pt = PtOut<OutT, NG>;
-    const Pt MU{reinterpret_cast<OutT*>(a.ptv) + (Pt::S == 1 ? (le * NG + g) * C::PT_VOL : le * NG * C::PT_VOL + g)};
+    using Pt = PtOut<NG>;
+    const Pt MU{a.ptv + le * NG * C::PT_VOL + g};
     const Pt FR = MU + M, T0 = FR + D * M, T1 = T0 + M * M, T2 = T1 + D * M * M;
     for (int i = 0; i < M; ++i) {
       put(MU, i, W * a.mass_coef * u[i].v);
@@ -229,24 +224,16 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
         }
       }
     if (C::VISC) {
-      // dG/dq contracted with the rows of Jinv (G is linear in q)
+      // dG/dq contracted with the rows of Jinv on both sides (G is linear in q)
       const ViscFactors<D> vf = visc_factors<D>(v);
       const PhysParams pv = visc_params_at(ph, v[M - 1]);
-      if constexpr (Pt::S > 1) {  // on both sides
 #pragma unroll 1
-        for (int rr = 0; rr < D * (D + 1); ++rr) {
-          double c2[D];
-          jinv_row<D>(Jinv, rr % (D + 1), c2);
-          visc_jac_pair<D>(vf, Jinv + rr / (D + 1) * D, c2, pv, [&](int i, int l, double val) {
-            put(T2, (rr * (M - 1) + i - 1) * (M - 1) + l - 1, -W * val);
-          });
-        }
-      } else {
-#pragma unroll 1
-        for (int r = 0; r < D; ++r)
-          visc_jac_dir<D>(vf, Jinv + r * D, pv, [&](int i, int l, int k, double val) {
-            put(T2, ((r * M + i) * M + l) * D + k, -W * val);
-          });
+      for (int rr = 0; rr < D * (D + 1); ++rr) {
+        double c2[D];
+        jinv_row<D>(Jinv, rr % (D + 1), c2);
+        visc_jac_pair<D>(vf, Jinv + rr / (D + 1) * D, c2, pv, [&](int i, int l, double val) {
+          put(T2, (rr * (M - 1) + i - 1) * (M - 1) + l - 1, -W * val);
+        });
       }
     }
   } else if (tid < NG + NF * NGF) {
@@ -342,10 +329,8 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
     prim_of_v<D>(vd, ph.gamma, rv, velv, pv);
     cons_and_flux<D>(rv, velv, pv, ph.gamma, (Dual<M>*)nullptr, Fv);
     bad = bad || !(rv.v > 0.0) || !(pv.v > 0.0);
-    using Pt = PtOut<OutT, NF * NGF>;
-    const int pf = f * NGF + gf;
-    const Pt HF{reinterpret_cast<OutT*>(a.ptf) +
-                (Pt::S == 1 ? (le * NF * NGF + pf) * C::PT_FACE : le * NF * NGF * C::PT_FACE + pf)};
+    using Pt = PtOut<NF * NGF>;
+    const Pt HF{a.ptf + le * NF * NGF * C::PT_FACE + f * NGF + gf};
     const Pt U0 = HF + M, U1 = U0 + M * M, U2 = U1 + M * M;
     Dual<M> gn[M];  // ghat = G(v, q) . n (Eq. numericalFluxNS_1): value and d/dv
     for (int i = 0; i < M; ++i) gn[i] = vd[0] * 0.0;
@@ -368,17 +353,13 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
       const double* vs = ph.gflux == 1 ? v : vh;
       const ViscFactors<D> vf = visc_factors<D>(vs);
       const PhysParams pvs = visc_params_at(ph, vs[M - 1]);
-      if constexpr (Pt::S > 1) {
 #pragma unroll 1
-        for (int r = 0; r <= D; ++r) {
-          double c2[D];
-          jinv_row<D>(Jinv, r, c2);
-          visc_jac_pair<D>(vf, n, c2, pvs, [&](int i, int l, double val) {
-            put(U2, (r * (M - 1) + i - 1) * (M - 1) + l - 1, Wf * val);
-          });
-        }
-      } else {
-        visc_jac_dir<D>(vf, n, pvs, [&](int i, int l, int k, double val) { put(U2, (i * M + l) * D + k, Wf * val); });
+      for (int r = 0; r <= D; ++r) {
+        double c2[D];
+        jinv_row<D>(Jinv, r, c2);
+        visc_jac_pair<D>(vf, n, c2, pvs, [&](int i, int l, double val) {
+          put(U2, (r * (M - 1) + i - 1) * (M - 1) + l - 1, Wf * val);
+        });
       }
     }
   }
@@ -386,13 +367,13 @@ __global__ void __launch_bounds__(128) k_pointwise(AssembleArgs a, DevTables T, 
 }
 
 // k_pointwise with the stabilization matrix the physics selects
-template <class C, class OutT = double>
+template <class C>
 void launch_pointwise(const AssembleArgs& a, const DevTables& T, const PhysParams& ph, cudaStream_t s) {
   const int threads = ((C::NG + C::NF * C::NGF + 31) / 32) * 32;
   if (ph.stab == 1)
-    k_pointwise<C, OutT, true><<<(unsigned)a.ne, threads, 0, s>>>(a, T, ph);
+    k_pointwise<C, true><<<(unsigned)a.ne, threads, 0, s>>>(a, T, ph);
   else
-    k_pointwise<C, OutT, false><<<(unsigned)a.ne, threads, 0, s>>>(a, T, ph);
+    k_pointwise<C, false><<<(unsigned)a.ne, threads, 0, s>>>(a, T, ph);
 }
 
 // ------------------------------------------------------------------------------------

@@ -1,8 +1,11 @@
-// Dispatch of the mixed-precision assemble + condense (asm_tc.cuh, condense_tc.cuh).
+// Dispatch of the mixed-precision assemble + condense (asm_t5.cuh, condense_tc.cuh).
 #include <algorithm>
+#include <array>
+#include <map>
+#include <set>
 #include <vector>
 
-#include "asm_tc.cuh"
+#include "asm_t5.cuh"
 #include "condense_t5.cuh"
 #include "condense_tc.cuh"
 #include "ctx.hpp"
@@ -13,63 +16,271 @@ namespace {
 
 constexpr int kSlices = 6;  // exact bf16 slices per operand in every tensor-core product
 
-int ensure_df_tables(hdg_ctx* ctx) {
-  if (ctx->d_tab_df) return HDG_OK;
-  // double-float copies of the reference tables, converted on the device-independent host
-  const size_t n_total = ctx->tab_size;
-  std::vector<double> h(n_total);
-  HDG_CK(cudaMemcpy(h.data(), ctx->d_tab, sizeof(double) * n_total, cudaMemcpyDeviceToHost));
-  std::vector<float> hd(2 * n_total);
-  for (size_t i = 0; i < n_total; ++i) {
-    float hi = (float)h[i];
-    float lo = (float)(h[i] - (double)hi);
-    hd[2 * i] = hi;
-    hd[2 * i + 1] = lo;
-  }
-  HDG_CK(cudaMalloc(&ctx->d_tab_df, sizeof(float) * hd.size()));
-  HDG_CK(cudaMemcpy(ctx->d_tab_df, hd.data(), sizeof(float) * hd.size(), cudaMemcpyHostToDevice));
-  return HDG_OK;
-}
+}  // namespace
 
-// One compiled shape of the assembly products: MTC row tiles (16 MTC rows) per CTA, NJW
-// column tiles per warp.
-struct AsmVariant {
-  int mtc, njw, threads;
-  void (*run_vol)(const AssembleArgs&, const DevTablesDF&, cudaStream_t);
-  void (*run_face)(const AssembleArgs&, const DevTables&, const DevTablesDF&, cudaStream_t);
-  int (*set_attr)();
-  void run(const AssembleArgs& a, const DevTables& T, const DevTablesDF& TD, cudaStream_t s) const {
-    run_vol(a, TD, s);
-    run_face(a, T, TD, s);
+// The assembly's constant operand and its schedule (asm_t5.cuh), built on the first mixed call of a context.
+struct T5Plan {
+  T5Prog prog[2] = {};  // rows with a viscous part, rows without
+  int nplane = 0;
+  df2* planes = nullptr;
+  std::vector<void*> bufs;
+  ~T5Plan() {
+    for (void* b : bufs) cudaFree(b);
   }
 };
 
-template <class C, int MTC, int NJW>
-void run_vol(const AssembleArgs& a, const DevTablesDF& TD, cudaStream_t s) {
-  using Q = AsmTC<C, kSlices, MTC, NJW>;
-  k_asm_vol_tc<C, kSlices, MTC, NJW><<<dim3(Q::NPASS, (unsigned)a.ne), Q::NTH, Q::vol_bytes, s>>>(a, TD);
-}
+void t5_plan_free(void* p) { delete static_cast<T5Plan*>(p); }
 
-template <class C, int MTC, int NJW>
-void run_face(const AssembleArgs& a, const DevTables& T, const DevTablesDF& TD, cudaStream_t s) {
-  using Q = AsmTC<C, kSlices, MTC, NJW>;
-  k_asm_face_tc<C, kSlices, MTC, NJW><<<dim3(Q::NFCTA, (unsigned)a.ne), Q::NTH, Q::face_bytes, s>>>(a, T, TD);
-}
+namespace {
 
-template <class C, int MTC, int NJW>
-int set_products_attr() {
-  using Q = AsmTC<C, kSlices, MTC, NJW>;
-  HDG_CK(cudaFuncSetAttribute(k_asm_vol_tc<C, kSlices, MTC, NJW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Q::vol_bytes));
-  HDG_CK(cudaFuncSetAttribute(k_asm_face_tc<C, kSlices, MTC, NJW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Q::face_bytes));
+template <class T>
+int t5_upload(T5Plan& pl, const std::vector<T>& v, T** out) {
+  HDG_CK(cudaMalloc(out, sizeof(T) * std::max<size_t>(1, v.size())));
+  pl.bufs.push_back(*out);
+  if (!v.empty()) HDG_CK(cudaMemcpy(*out, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
   return HDG_OK;
 }
 
-template <class C, int MTC, int NJW>
-AsmVariant make_variant() {
-  return AsmVariant{MTC, NJW, AsmTC<C, kSlices, MTC, NJW>::NTH, &run_vol<C, MTC, NJW>, &run_face<C, MTC, NJW>,
-                    &set_products_attr<C, MTC, NJW>};
+// One row program: its entries of k in chunks of at most 128, and per chunk the groups of up to 32
+// columns that use the same steps of 16 entries.
+template <class C>
+int t5_program(hdg_ctx* ctx, T5Plan& pl, bool viscous, T5Prog& P, cudaStream_t s) {
+  constexpr int D = C::D, M = C::M, NP = C::NP, NFN = C::NFN, NF = C::NF, NG = C::NG, NGF = C::NGF, NV = C::NV,
+                NT = C::NT, NTN = NF * NFN;
+  const RefElement& ref = ctx->mesh->m.ref;
+  std::vector<int> pairs;
+  for (int i = 0; i < M; ++i)
+    for (int l = 0; l < M; ++l)
+      if ((C::VISC && i > 0 && l > 0) == viscous) pairs.push_back(i << 8 | l);
+  P = T5Prog{};
+  if (pairs.empty()) return HDG_OK;
+  P.rpe = (int)pairs.size();
+  P.ept = 128 / P.rpe;
+  // operators in order: faces first (the running sums of A', B' end with the volume); short ones share a step
+  std::vector<std::vector<T5Entry>> chunks;
+  std::vector<T5Entry> cur;
+  auto block = [&](int kind, int f, int r, int r2, int n, int pt0) {
+    if (n > 8)
+      while (cur.size() % 16) cur.push_back({T5_PAD, 0, 0, 0, 0});
+    if (cur.size() + n > 128) {
+      chunks.push_back(cur);
+      cur.clear();
+    }
+    for (int g = 0; g < n; ++g) cur.push_back({(short)kind, (short)f, (short)r, (short)r2, pt0 + g});
+  };
+  constexpr int face_room = (D + 3) * (NGF > 8 ? (NGF + 15) / 16 * 16 : NGF) + (NGF > 8 ? 15 : 0);
+  static_assert(face_room <= 128 + 15, "a face's operators share one chunk: its C', D' entries are one product");
+  for (int f = 0; f < NF; ++f) {
+    if (cur.size() + face_room > 128) {
+      if (!cur.empty()) chunks.push_back(cur);
+      cur.clear();
+    }
+    block(T5_U0, f, 0, 0, NGF, f * NGF);
+    if (viscous)
+      for (int r2 = 0; r2 <= D; ++r2) block(T5_U2, f, 0, r2, NGF, f * NGF);
+    block(T5_U1, f, 0, 0, NGF, f * NGF);
+  }
+  chunks.push_back(cur);
+  cur.clear();
+  block(T5_T0, 0, 0, 0, NG, 0);
+  for (int r = 0; r < D; ++r) block(T5_T1, 0, r, 0, NG, 0);
+  if (viscous)
+    for (int r2 = 0; r2 <= D; ++r2)
+      for (int r = 0; r < D; ++r) block(T5_T2, 0, r, r2, NG, 0);
+  chunks.push_back(cur);
+  P.nchunk = (int)chunks.size();
+  std::vector<int> cstep(1, 0);
+  std::vector<T5Entry> ent;
+  for (auto& c : chunks) {
+    cstep.push_back(cstep.back() + (int)(c.size() + 15) / 16);
+    c.resize(128, {T5_PAD, 0, 0, 0, 0});
+    ent.insert(ent.end(), c.begin(), c.end());
+  }
+  P.nsteps = cstep.back();
+  // columns
+  struct Col {
+    T5ColDesc d;
+    int plane, direct;
+  };
+  std::vector<char> on_face(NF * NP, 0);
+  for (int f = 0; f < NF; ++f)
+    for (int c = 0; c < NFN; ++c) on_face[f * NP + ref.face_nodes[f][c]] = 1;
+  const int nplane = NP * NP + NP * NTN;
+  std::vector<int> fin(nplane);  // A' then B'
+  std::vector<Col> all;
+  for (int a = 0; a < NP; ++a) {
+    for (int j = 0; j < NP; ++j) {
+      fin[a * NP + j] = a * M * NV + j * M;
+      all.push_back({{T5_COL_A, 0, (short)a, (short)j, 0, 0}, a * NP + j, -1});
+    }
+    for (int f = 0; f < NF; ++f)
+      for (int c = 0; c < NFN; ++c) {
+        const int p = NP * NP + a * NTN + f * NFN + c;
+        fin[p] = 1 << 28 | (a * M * NT + (f * NFN + c) * M);
+        all.push_back({{T5_COL_B, (short)f, (short)a, (short)c, 0, 0}, p, -1});
+      }
+  }
+  for (int f = 0; f < NF; ++f)
+    for (int c = 0; c < NFN; ++c) {
+      const int node = ref.face_nodes[f][c], row = (f * NFN + c) * M;
+      for (int j = 0; j < NP; ++j)
+        all.push_back({{T5_COL_FI, (short)f, (short)c, (short)j, 0, 0}, node * NP + j, 2 << 28 | (row * NV + j * M)});
+      for (int f2 = 0; f2 < NF; ++f2)
+        for (int c2 = 0; c2 < NFN; ++c2)
+          all.push_back({{T5_COL_FT, (short)f, (short)c, (short)c2, (short)f2, 0},
+                         NP * NP + node * NTN + f2 * NFN + c2, 3 << 28 | (row * NT + (f2 * NFN + c2) * M)});
+    }
+  auto uses = [&](const T5ColDesc& d, const T5Entry& e) {
+    switch (d.kind) {
+      case T5_COL_A: return e.kind == T5_T0 || e.kind == T5_T1 || (e.kind == T5_T2 && e.r2 < D);
+      case T5_COL_B: return e.kind == T5_T2 && e.r2 == (d.f ? d.f - 1 : D);
+      case T5_COL_FI:
+        return e.f == d.f && ((e.kind == T5_U0 && on_face[d.f * NP + d.j]) || (e.kind == T5_U2 && e.r2 < D));
+      default: return e.f == d.f && ((e.kind == T5_U1 && d.f2 == d.f) || (e.kind == T5_U2 && e.r2 == (d.f2 ? d.f2 - 1 : D)));
+    }
+  };
+  // jobs: columns of one kind and one set of steps, the planes' first additions before the others of a chunk and
+  // their last ones behind; a plane fixes its quarter of a group and comes once in it at most
+  auto quarter = [&](int p) { return p < NP * NP ? (p / NP + p % NP) & 3 : ((p - NP * NP) / NTN + (p - NP * NP) % NTN) & 3; };
+  std::vector<std::vector<int>> masks(P.nchunk, std::vector<int>(all.size(), 0));
+  std::vector<int> left(nplane, 0), seen(nplane, 0);
+  std::vector<char> written(all.size(), 0);
+  for (int ch = 0; ch < P.nchunk; ++ch)
+    for (size_t k = 0; k < all.size(); ++k) {
+      int mask = 0;
+      for (int x = 0; x < 128; ++x)
+        if (chunks[ch][x].kind != T5_PAD && uses(all[k].d, chunks[ch][x])) mask |= 1 << (x / 16);
+      masks[ch][k] = mask;
+      if (mask) {
+        written[k] = 1;
+        ++left[all[k].plane];
+      }
+    }
+  const T5Col none = {nplane * 128 * (int)sizeof(df2), -1, 0.f, -1};
+  std::vector<int> jobs, wstep;
+  std::vector<T5Col> cols;
+  std::vector<T5ColDesc> desc;
+  int wsteps = 0;
+  std::set<int> before;  // planes of the job before
+  for (int ch = 0; ch < P.nchunk; ++ch) {
+    std::map<std::array<int, 4>, std::vector<int>> groups;  // (not first, last, kind, steps)
+    for (size_t k = 0; k < all.size(); ++k)
+      if (masks[ch][k]) {
+        const int p = all[k].plane;
+        groups[{seen[p] ? 1 : 0, --left[p] ? 0 : 1, all[k].d.kind, masks[ch][k]}].push_back((int)k);
+        ++seen[p];
+      }
+    for (auto& gr : groups) {
+      std::vector<int> rest = gr.second;
+      while (!rest.empty()) {
+        int job = gr.first[3] | ch << 8 | (gr.first[0] ? 0 : T5_FIRST) | (gr.first[1] ? T5_LAST : 0) |
+                  gr.first[2] << T5_KIND;
+        wstep.push_back(wsteps);
+        for (int m = gr.first[3]; m; m &= m - 1) ++wsteps;
+        cols.resize((jobs.size() + 1) * kT5Cols, none);
+        desc.resize((jobs.size() + 1) * kT5Cols, {T5_COL_NONE, 0, 0, 0, 0, 0});
+        int fill[4] = {0, 0, 0, 0};
+        std::set<int> taken;
+        std::vector<int> later;
+        for (int k : rest) {
+          const Col& c = all[k];
+          const int h = quarter(c.plane);
+          if (fill[h] == kT5Q || taken.count(c.plane)) {
+            later.push_back(k);
+            continue;
+          }
+          taken.insert(c.plane);
+          if (before.count(c.plane)) job |= T5_HAZARD;
+          const size_t at = jobs.size() * kT5Cols + h * kT5Q + fill[h]++;
+          cols[at] = {c.plane * 128 * (int)sizeof(df2), c.direct < 0 ? -1 : (c.direct & 0xfffffff) * 8, 0.f,
+                      (fin[c.plane] & 0xfffffff) * 8};
+          desc[at] = c.d;
+        }
+        rest.swap(later);
+        before.swap(taken);
+        jobs.push_back(job);
+      }
+    }
+    jobs.back() |= T5_CLOSES;
+  }
+  std::vector<int> zero;  // entries that vanish for these pairs
+  for (int p = 0; p < nplane; ++p)
+    if (!seen[p]) zero.push_back(fin[p]);
+  for (size_t k = 0; k < all.size(); ++k)
+    if (!written[k] && all[k].direct >= 0) zero.push_back(all[k].direct);
+  for (int k = 0; k < 2 * kT5Cols; ++k) cols.push_back(none);
+  P.njob = (int)jobs.size();
+  P.nzero = (int)zero.size();
+  pl.nplane = nplane;
+  int *dj, *dc, *dp, *dws, *dz;
+  T5Entry* de;
+  T5ColDesc* dd;
+  unsigned char* dw;
+  int rc;
+  if ((rc = t5_upload(pl, jobs, &dj)) || (rc = t5_upload(pl, cols, &P.cols)) || (rc = t5_upload(pl, desc, &dd)) ||
+      (rc = t5_upload(pl, ent, &de)) || (rc = t5_upload(pl, cstep, &dc)) || (rc = t5_upload(pl, pairs, &dp)) ||
+      (rc = t5_upload(pl, wstep, &dws)) || (rc = t5_upload(pl, zero, &dz)))
+    return rc;
+  P.wstep = dws;
+  P.zero = dz;
+  HDG_CK(cudaMalloc(&dw, (size_t)wsteps * kT5Slices * kT5BTile));
+  pl.bufs.push_back(dw);
+  P.jobs = dj;
+  P.ent = de;
+  P.cstep = dc;
+  P.pairs = dp;
+  P.W = dw;
+  k_t5_weights<C><<<P.njob, 256, 0, s>>>(ctx->T, P, dd, dw);
+  HDG_CK(cudaGetLastError());
+  return HDG_OK;
+}
+
+template <class C>
+int t5_plan(hdg_ctx* ctx, cudaStream_t s) {
+  if (ctx->t5_plan) return HDG_OK;
+  auto* pl = new T5Plan();
+  int rc = HDG_OK;
+  if ((rc = t5_program<C>(ctx, *pl, true, pl->prog[0], s)) || (rc = t5_program<C>(ctx, *pl, false, pl->prog[1], s))) {
+    delete pl;
+    return rc;
+  }
+  if (cudaMalloc(&pl->planes, sizeof(df2) * (size_t)ctx->num_sms * (pl->nplane + 1) * 128) != cudaSuccess) {
+    delete pl;
+    return cuda_fail(cudaGetLastError(), "cudaMalloc (assembly planes)");
+  }
+  pl->bufs.push_back(pl->planes);
+  if (pl->prog[0].njob + pl->prog[1].njob > kT5MaxJobs) {
+    delete pl;
+    set_error("assemble_condense: the assembly's schedule is longer than its table");
+    return HDG_ERR_UNSUPPORTED;
+  }
+  // later calls may come on other streams
+  if (cudaStreamSynchronize(s) != cudaSuccess) {
+    delete pl;
+    return cuda_fail(cudaGetLastError(), "assembly operands");
+  }
+  ctx->t5_plan = pl;
+  return HDG_OK;
+}
+
+// tiles and scratch bytes (slices, row exponents) of a program over n elements
+int64_t t5_tiles(const T5Prog& P, int64_t n) { return P.ept ? (n + P.ept - 1) / P.ept : 0; }
+size_t t5_slice_bytes(const T5Prog& P, int64_t n) {
+  return (size_t)t5_tiles(P, n) * P.nsteps * kT5Slices * kT5ATile;
+}
+size_t t5_exp_bytes(const T5Prog& P, int64_t n) { return (size_t)t5_tiles(P, n) * P.nchunk * 128 * sizeof(int); }
+
+template <class C>
+void run_asm_t5(hdg_ctx* ctx, const T5Plan& pl, const T5Prog (&pr)[2], const AssembleArgs& a, cudaStream_t s) {
+  {
+    LaunchScope ls(ctx, HDG_KERNEL_MIXED_OPERATORS, s);
+    for (const T5Prog& P : pr)
+      if (P.ntile)
+        k_t5_rows<C><<<dim3((unsigned)P.ntile, (unsigned)P.nchunk), 256, 0, s>>>(a, P, const_cast<unsigned char*>(P.T));
+  }
+  LaunchScope ls(ctx, HDG_KERNEL_MIXED_ASSEMBLE, s);
+  const int grid = std::min(ctx->num_sms, pr[0].ntile + pr[1].ntile);
+  k_asm_t5<C><<<grid, kT5Threads, kT5Smem, s>>>(a, pr[0], pr[1], pl.planes, pl.nplane);
 }
 
 // One compiled shape of the condensation kernel, with the prep kernel that lays out its operands.
@@ -122,20 +333,23 @@ int time_launch(cudaStream_t s, F launch, float* ms) {
 template <class C>
 int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* hist, double mass_coef, double* S,
               double* g, double* recov, double* R, int32_t* status, cudaStream_t s) {
-  int rc = ensure_df_tables(ctx);
-  if (rc) return rc;
+  if (!ctx->num_sms) HDG_CK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  if (int rc = t5_plan<C>(ctx, s)) return rc;
+  const T5Plan& pl = *static_cast<T5Plan*>(ctx->t5_plan);
+  T5Prog pr[2] = {pl.prog[0], pl.prog[1]};
   using TC = CondTC<C, 256, kSlices>;
-  using AQ = AsmTC<C, kSlices, 2>;  // the operator slices do not depend on the row tiling
   const size_t per_pt = sizeof(double) * ((size_t)C::NG * C::PT_VOL + (size_t)C::NF * C::NGF * C::PT_FACE +
                                           (size_t)C::NV * C::NV + (size_t)C::NT * C::NV);
   const size_t slice_bytes = std::max(sizeof(uint4) * TC::slice_uint4, CondT5<C, kSlices>::slice_bytes);
-  const size_t per = per_pt + slice_bytes + sizeof(float) * TC::prep_floats + sizeof(uint2) * AQ::rb_u2;
+  const size_t per_rows = t5_slice_bytes(pr[0], 1024) / 1024 + t5_slice_bytes(pr[1], 1024) / 1024;
+  const size_t per = per_pt + slice_bytes + sizeof(float) * TC::prep_floats + per_rows;
   if (ctx->chunk == 0) {
     int64_t ch = std::min<int64_t>(ctx->E, 8192);
     while (ch > 256 && per * ch > ((size_t)16 << 30)) ch /= 2;
     ctx->chunk = ch;
   }
-  const size_t need = per * ctx->chunk + 1024;  // + room to align the slice, prep and operator scratch
+  size_t need = (per - per_rows) * ctx->chunk + 4096;  // + room to align the parts of the scratch
+  for (const T5Prog& P : pr) need += t5_slice_bytes(P, ctx->chunk) + t5_exp_bytes(P, ctx->chunk) + 1024;
   if (ctx->scr_bytes < need) {
     if (ctx->d_scr) cudaFree(ctx->d_scr);
     ctx->d_scr = nullptr;
@@ -143,16 +357,11 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     HDG_CK(cudaMalloc(&ctx->d_scr, need));
     ctx->scr_bytes = need;
   }
-  // compiled tile shapes of the assembly kernel (threads, volume points per tile)
-  const AsmVariant variants[] = {make_variant<C, 2, 4>(), make_variant<C, 4, 4>(), make_variant<C, 2, 2>(),
-                                 make_variant<C, 4, 2>()};
-  constexpr int NVAR = 4;
   const CondVariant cvariants[] = {make_cond_variant<C, 256>(), make_cond_variant<C, 512>(), make_cond_variant2<C>(),
                                    make_cond_variant_t5<C>()};
   constexpr int NCVAR = 4;
   if (!ctx->attr_mixed) {  // per context, hence per device
-    for (const AsmVariant& v : variants)
-      if (int rc2 = v.set_attr()) return rc2;
+    HDG_CK(cudaFuncSetAttribute(k_asm_t5<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kT5Smem));
     for (const CondVariant& v : cvariants) {
       HDG_CK(cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.smem));
       HDG_CK(cudaFuncSetAttribute(v.kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
@@ -166,14 +375,6 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     HDG_CK(cudaFuncSetAttribute(k_condense<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CondSmem<C>::bytes));
     ctx->attr_mixed = true;
   }
-  const df2* td = reinterpret_cast<const df2*>(ctx->d_tab_df);
-  DevTablesDF TD;
-  TD.Phi = td + (ctx->T.Phi - ctx->d_tab);
-  TD.dPhi = td + (ctx->T.dPhi - ctx->d_tab);
-  TD.PL = td + (ctx->T.PL - ctx->d_tab);
-  TD.PhiF = td + (ctx->T.PhiF - ctx->d_tab);
-  TD.dPhiF = td + (ctx->T.dPhiF - ctx->d_tab);
-  TD.PLF = td + (ctx->T.PLF - ctx->d_tab);
   AssembleArgs a{};
   a.V = V;
   a.Vhat = Vhat;
@@ -198,8 +399,14 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     a.oz = reinterpret_cast<uint4*>((p + 255) & ~(uintptr_t)255);
     const uintptr_t q = reinterpret_cast<uintptr_t>(a.oz) + ch * slice_bytes;
     a.prep = reinterpret_cast<float*>((q + 255) & ~(uintptr_t)255);
-    const uintptr_t r = reinterpret_cast<uintptr_t>(a.prep + ch * TC::prep_floats);
-    a.rb = reinterpret_cast<uint2*>((r + 255) & ~(uintptr_t)255);
+    uintptr_t r = reinterpret_cast<uintptr_t>(a.prep + ch * TC::prep_floats);
+    for (T5Prog& P : pr) {
+      r = (r + 255) & ~(uintptr_t)255;
+      P.T = reinterpret_cast<unsigned char*>(r);
+      r += t5_slice_bytes(P, ch);
+      P.erow = reinterpret_cast<int*>(r);
+      r += t5_exp_bytes(P, ch);
+    }
   }
   for (int64_t e0 = 0; e0 < ctx->E; e0 += ch) {
     a.e0 = e0;
@@ -211,84 +418,34 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     }
     {
       LaunchScope ls(ctx, HDG_KERNEL_POINTWISE, s);
-      launch_pointwise<C, df2>(a, ctx->T, ctx->ph, s);
+      launch_pointwise<C>(a, ctx->T, ctx->ph, s);
     }
     {
       LaunchScope ls(ctx, HDG_KERNEL_MIXED_OPERATORS, s);
-      k_asm_rb<C, kSlices, 2><<<(unsigned)a.ne, 256, 0, s>>>(a, ctx->T, TD);
+      k_residual<C><<<(unsigned)a.ne, 128, 0, s>>>(a, ctx->T);
     }
-    {
-      LaunchScope ls(ctx, HDG_KERNEL_MIXED_OPERATORS, s);
-      k_asm_residual<C><<<(unsigned)a.ne, 128, 0, s>>>(a, ctx->T);
-    }
-    if ((ctx->asm_variant < 0 || ctx->face_variant < 0 || ctx->cond_variant < 0) && a.ne >= 512) {
-      // autotune on this chunk: time every compiled shape (each rewrites the same outputs);
-      // the volume and face products are tuned separately (the faces add to the volume's
-      // output, so the volume runs again before each face trial)
-      if (ctx->asm_variant < 0) {
-        float best = 1e30f;
-        int best_i = 0;
-        for (int i = 0; i < NVAR; ++i) {
-          float ms = 0.f;
-          const AsmVariant& v = variants[i];
-          int rc = time_launch(s, [&] { v.run_vol(a, TD, s); }, &ms);
-          if (rc) return rc;
-          if (ms < best) {
-            best = ms;
-            best_i = i;
-          }
+    for (T5Prog& P : pr) P.ntile = (int)t5_tiles(P, a.ne);
+    if (ctx->cond_variant < 0 && a.ne >= 512) {
+      // autotune on this chunk: time every compiled shape of the condensation
+      float best = 1e30f;
+      int best_i = 0;
+      for (int i = 0; i < NCVAR; ++i) {
+        // the condensation overwrites its inputs: assemble again before each trial
+        run_asm_t5<C>(ctx, pl, pr, a, s);
+        const CondVariant& cv = cvariants[i];
+        cv.prep<<<(unsigned)a.ne, TC::PTH, TC::prep_bytes, s>>>(a);
+        float ms = 0.f;
+        int rc = time_launch(s, [&] { cv.kernel<<<cv.grid(a.ne), cv.threads, cv.smem, s>>>(a); }, &ms);
+        if (rc) return rc;
+        if (ms < best) {
+          best = ms;
+          best_i = i;
         }
-        ctx->asm_variant = best_i;
-        ctx->asm_variant_threads = variants[best_i].threads;
-        ctx->asm_variant_gt = 16 * variants[best_i].mtc;
       }
-      if (ctx->face_variant < 0) {
-        float best = 1e30f;
-        int best_i = 0;
-        for (int i = 0; i < NVAR; ++i) {
-          variants[ctx->asm_variant].run_vol(a, TD, s);
-          float ms = 0.f;
-          const AsmVariant& v = variants[i];
-          int rc = time_launch(s, [&] { v.run_face(a, ctx->T, TD, s); }, &ms);
-          if (rc) return rc;
-          if (ms < best) {
-            best = ms;
-            best_i = i;
-          }
-        }
-        ctx->face_variant = best_i;
-      }
-      if (ctx->cond_variant < 0) {
-        const AsmVariant& vv = variants[ctx->asm_variant];
-        const AsmVariant& vf = variants[ctx->face_variant];
-        float best = 1e30f;
-        int best_i = 0;
-        for (int i = 0; i < NCVAR; ++i) {
-          // the condensation overwrites its inputs: assemble again before each trial
-          vv.run_vol(a, TD, s);
-          vf.run_face(a, ctx->T, TD, s);
-          const CondVariant& cv = cvariants[i];
-          cv.prep<<<(unsigned)a.ne, TC::PTH, TC::prep_bytes, s>>>(a);
-          float ms = 0.f;
-          int rc = time_launch(s, [&] { cv.kernel<<<cv.grid(a.ne), cv.threads, cv.smem, s>>>(a); }, &ms);
-          if (rc) return rc;
-          if (ms < best) {
-            best = ms;
-            best_i = i;
-          }
-        }
-        ctx->cond_variant = best_i;
-        ctx->cond_variant_threads = cvariants[best_i].threads;
-      }
+      ctx->cond_variant = best_i;
+      ctx->cond_variant_threads = cvariants[best_i].threads;
     }
-    {
-      LaunchScope ls(ctx, HDG_KERNEL_MIXED_ASSEMBLE, s);
-      variants[ctx->asm_variant < 0 ? 0 : ctx->asm_variant].run_vol(a, TD, s);
-    }
-    {
-      LaunchScope ls(ctx, HDG_KERNEL_MIXED_FACE, s);
-      variants[ctx->face_variant < 0 ? 0 : ctx->face_variant].run_face(a, ctx->T, TD, s);
-    }
+    run_asm_t5<C>(ctx, pl, pr, a, s);
     if (int rc_b = boundary_patch(ctx, a, HDG_PREC_MIXED, s)) return rc_b;
     const CondVariant& cv = cvariants[ctx->cond_variant < 0 ? 0 : ctx->cond_variant];
     {
@@ -301,14 +458,9 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     }
     if (ctx->refine_fallback) {
       // blocks whose refinement missed its tolerance (or whose condensation gave up a wait) are
-      // recomputed by the FP64 kernels (the chunk's scratch is free again); every other CTA
-      // returns at once
+      // recomputed by the FP64 kernels from the same point tensors; every other CTA returns at once
       AssembleArgs f = a;
       f.only_flag = HDG_STATUS_REFINE | HDG_STATUS_TIMEOUT;
-      {
-        LaunchScope ls(ctx, HDG_KERNEL_POINTWISE, s);
-        launch_pointwise<C>(f, ctx->T, ctx->ph, s);
-      }
       {
         LaunchScope ls(ctx, HDG_KERNEL_ASSEMBLE, s);
         k_assemble<C><<<(unsigned)a.ne, AsmSmem<C>::NTH, AsmSmem<C>::bytes, s>>>(f, ctx->T);

@@ -369,10 +369,6 @@ int hdg_ctx_create(hdg_mesh_t mesh, const hdg_physics* phys, int device, hdg_ctx
   c->scheme = m.scheme == HDG_SCHEME_HDG ? 0 : 1;
   c->n_tnodes = m.scheme == HDG_SCHEME_HDG ? m.nFaces * m.ref.Nf : m.n_edg;
   c->ntrace = c->n_tnodes * c->M;
-  if (const char* av = std::getenv("HDG_ASM_VARIANT")) {  // force a tile shape (tests)
-    long v = std::strtol(av, nullptr, 10);
-    if (v >= 0 && v < 4) c->asm_variant = c->face_variant = (int)v;
-  }
   if (const char* cv = std::getenv("HDG_COND_VARIANT")) {  // force a condensation shape (tests)
     long v = std::strtol(cv, nullptr, 10);
     if (v >= 0 && v < 4) c->cond_variant = (int)v;
@@ -509,7 +505,7 @@ int hdg_ctx_create(hdg_mesh_t mesh, const hdg_physics* phys, int device, hdg_ctx
 void hdg_ctx_destroy(hdg_ctx_t c) {
   if (!c) return;
   DeviceGuard guard(c->device);
-  void* bufs[] = {c->d_tab, c->d_tab_df, c->d_itab, c->d_tgidx, c->d_geo, c->d_fs_elem, c->d_fs_loc, c->d_scr,
+  void* bufs[] = {c->d_tab, c->d_itab, c->d_tgidx, c->d_geo, c->d_fs_elem, c->d_fs_loc, c->d_scr,
                   c->d_sw, c->d_pc, c->d_dense, c->d_dpiv, c->d_red, c->d_S,
                   c->d_g, c->d_recov, c->d_R, c->d_dV, c->d_dVh, c->d_status, c->d_hist, c->d_V0,
                   c->d_Vh0, c->d_feat, c->d_pred, c->d_dirk, c->d_ent, c->d_tr_ptr, c->d_tr_occ, c->d_pcn,
@@ -537,6 +533,7 @@ void hdg_ctx_destroy(hdg_ctx_t c) {
     cudaEventDestroy(r.a);
     cudaEventDestroy(r.b);
   }
+  hdg::t5_plan_free(c->t5_plan);
   hdg::pclass_free(c->pm);
   delete c;
 }

@@ -44,7 +44,6 @@ struct hdg_ctx {
   // device tables
   double* d_tab = nullptr;
   size_t tab_size = 0;       // doubles in d_tab
-  float* d_tab_df = nullptr; // the same tables as double-float pairs (mixed form)
   int* d_itab = nullptr;
   hdg::DevTables T{};
   int* d_tgidx = nullptr;    // [E][NF][NFN] canonical global face node of each local face node
@@ -55,9 +54,7 @@ struct hdg_ctx {
   int64_t chunk = 0;
   double* d_scr = nullptr;
   size_t scr_bytes = 0;
-  // autotuned tile shape of the mixed assembly (-1: not chosen yet)
-  int asm_variant = -1, asm_variant_threads = 0, asm_variant_gt = 0;  // volume products
-  int face_variant = -1;                                              // face products
+  void* t5_plan = nullptr;  // mixed assembly: constant operand and schedule (assemble_mixed.cu)
   int cond_variant = -1, cond_variant_threads = 0;  // mixed condensation shape
   // solver scratch
   double* d_sw = nullptr;    // GMRES / matvec workspace
@@ -201,6 +198,7 @@ struct AssembleArgs;  // assemble_fp64.cuh
 // element assembly left in R_t, C and D (boundary.cu); precision selects the output form
 int boundary_patch(hdg_ctx* ctx, const AssembleArgs& a, int precision, cudaStream_t s);
 // int rho s and the physical entropy production of Eq. PiS added into acc[0], acc[1]
+void t5_plan_free(void* plan);  // assemble_mixed.cu
 int entropy_terms(hdg_ctx* ctx, const double* V, const double* Vhat, double* acc, cudaStream_t s);
 
 // trace-space and element helpers (trace.cu)

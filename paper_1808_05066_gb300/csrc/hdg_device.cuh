@@ -36,8 +36,8 @@ struct Cfg {
   static constexpr int NR = VISC ? D + 1 : 1;  // volume right operators: value (+ grad)
   static constexpr int NRF = VISC ? D + 2 : 2; // face right operators: v, vhat (+ grad)
   // per-point tensors written by the pointwise kernel
-  static constexpr int PT_VOL = M + D * M + M * M + D * M * M + (VISC ? D * M * M * D : 0);
-  static constexpr int PT_FACE = M + 2 * M * M + (VISC ? M * M * D : 0);
+  static constexpr int PT_VOL = M + D * M + M * M + D * M * M + (VISC ? D * (D + 1) * (M - 1) * (M - 1) : 0);
+  static constexpr int PT_FACE = M + 2 * M * M + (VISC ? (D + 1) * (M - 1) * (M - 1) : 0);
 };
 
 struct PhysParams {
@@ -369,69 +369,14 @@ HDG_DEVI ViscFactors<D> visc_factors(const double* v) {
   return f;
 }
 
-// sum_j c_j dG_ij/dq_lk for one vector c: the viscous flux (Eq. viscFlux) is linear in q, and
-// differentiating it by hand gives, with V_a = -w_a/v_m, A_a = w_a/v_m^2 and the Kronecker
-// delta d,
-//   momentum i = 1+a, l = 1+b:    mu/v_m (d_ab c_k + d_ak c_b - 2/3 d_bk c_a)
-//   momentum i = 1+a, l = m-1:   -mu (A_a c_k + d_ak c.A - 2/3 A_k c_a)
-//   energy   i = m-1, l = 1+b:    mu/v_m (V_b c_k + V_k c_b - 2/3 d_bk c.V)
-//   energy   i = m-1, l = m-1:   -mu (V.A c_k + V_k c.A - 2/3 A_k c.V) - kappa/(c_v v_m^2) c_k
-// and zero for i = 0 or l = 0. emit(i, l, k, value) receives every entry; the deltas are
-// branches on unrolled indices, so no arithmetic is spent on the vanishing terms.
-template <int D, class Emit>
-HDG_DEVI void visc_jac_dir(const ViscFactors<D>& f, const double* c, const PhysParams& ph, Emit emit) {
-  constexpr int M = D + 2;
-  constexpr double t3 = 2.0 / 3.0;
-  double cA = c[0] * f.A[0], cV = c[0] * f.vel[0], VA = f.vel[0] * f.A[0];
-#pragma unroll
-  for (int j = 1; j < D; ++j) {
-    cA += c[j] * f.A[j];
-    cV += c[j] * f.vel[j];
-    VA += f.vel[j] * f.A[j];
-  }
-  const double mi = ph.mu * f.ivm, kc = (ph.kappa / ph.cv) * f.ivm2;
-#pragma unroll
-  for (int k = 0; k < D; ++k) {
-#pragma unroll
-    for (int l = 0; l < M; ++l) emit(0, l, k, 0.0);
-#pragma unroll
-    for (int i = 1; i < M; ++i) emit(i, 0, k, 0.0);
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-#pragma unroll
-      for (int b = 0; b < D; ++b) {
-        double s = 0.0;
-        bool any = false;
-        if (a == b) {
-          s = c[k];
-          any = true;
-        }
-        if (a == k) {
-          s = any ? s + c[b] : c[b];
-          any = true;
-        }
-        if (b == k) {
-          s = any ? s - t3 * c[a] : -t3 * c[a];
-          any = true;
-        }
-        emit(1 + a, 1 + b, k, any ? mi * s : 0.0);
-      }
-      double s = f.A[a] * c[k] - t3 * f.A[k] * c[a];
-      if (a == k) s += cA;
-      emit(1 + a, M - 1, k, -ph.mu * s);
-    }
-#pragma unroll
-    for (int b = 0; b < D; ++b) {
-      double s = f.vel[b] * c[k] + f.vel[k] * c[b];
-      if (b == k) s -= t3 * cV;
-      emit(M - 1, 1 + b, k, mi * s);
-    }
-    emit(M - 1, M - 1, k, -ph.mu * (VA * c[k] + f.vel[k] * cA - t3 * f.A[k] * cV) - kc * c[k]);
-  }
-}
-
-// sum_jk c_j c2_k dG_ij/dq_lk: visc_jac_dir contracted with a second vector, for i, l >= 1 (the
-// other entries vanish). emit(i, l, value).
+// sum_jk c_j c2_k dG_ij/dq_lk for two vectors: the viscous flux (Eq. viscFlux) is linear in q, and
+// differentiating it by hand gives, with V_a = -w_a/v_m, A_a = w_a/v_m^2 and i, l >= 1 (the entries
+// with i = 0 or l = 0 vanish),
+//   momentum a, b:    mu/v_m (d_ab c.c2 + c2_a c_b - 2/3 c_a c2_b)
+//   momentum a, m-1: -mu (A_a c.c2 + c2_a c.A - 2/3 c2.A c_a)
+//   energy m-1, b:    mu/v_m (V_b c.c2 + c2.V c_b - 2/3 c2_b c.V)
+//   energy m-1, m-1: -mu (V.A c.c2 + c2.V c.A - 2/3 c2.A c.V) - kappa/(c_v v_m^2) c.c2
+// emit(i, l, value) receives every entry.
 template <int D, class Emit>
 HDG_DEVI void visc_jac_pair(const ViscFactors<D>& f, const double* c, const double* c2, const PhysParams& ph,
                             Emit emit) {

@@ -29,11 +29,12 @@ HDG_DEVI unsigned oz_pack2(float lo, float hi) {
   return *reinterpret_cast<unsigned*>(&v);
 }
 
-// Exponent E with max|x| < 2^E (0 for an all-zero row), and the slicing scale 2^(8-E).
+// Exponent E with max|x| < 2^E (0 for an all-zero row), and the slicing scale 2^(8-E). E stays above
+// -100: the scale of a row of subnormal numbers would overflow.
 HDG_DEVI int oz_exponent(float amax) {
   int E = 0;
   if (amax > 0.f) frexpf(amax, &E);
-  return E;
+  return E > -100 ? E : -100;
 }
 HDG_DEVI float oz_scale(int E) { return ldexpf(1.f, 8 - E); }  // per row / column, not per entry
 
