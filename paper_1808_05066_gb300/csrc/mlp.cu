@@ -158,172 +158,288 @@ HDG_DEVI void mlp_split2(float x0, float x1, unsigned& hi, unsigned& lo) {
   lo = *reinterpret_cast<const unsigned*>(&l);
 }
 
-constexpr int kTcLd = MAXH + 4;  // row stride (floats) of a warp's activation tile
-
-// One layer of 16 samples: out[16][N] = f(in[16][K] W^T + b), W [N][K] row-major (bf16, shared).
-// Fragment layout of m16n8k16 (g = lane / 4, t = lane % 4): A rows g, g + 8 at columns 2t, 2t + 1
-// and 2t + 8, 2t + 9 of the k tile; B (col-major) rows 2t, 2t + 1 and 2t + 8, 2t + 9 of column g;
-// C rows g, g + 8 at columns 2t, 2t + 1.
-template <int K, int N, bool TANH>
-HDG_DEVI void mlp_layer_tc(const __nv_bfloat16* W, const __nv_bfloat16* bias, const float* in, float* out,
-                           int lane) {
+// One layer of a warp's 16 samples, out[16][N] = f(in[16][K] W^T + b), in and out as A fragments of m16n8k16 split into
+// hi and lo (g = lane / 4, t = lane % 4: rows g, g + 8 at columns 2t, 2t + 1 and 2t + 8, 2t + 9 of each k tile). The
+// accumulators of two neighbouring 8-column tiles hold exactly the entries of the next layer's k tile in its
+// fragment's places, so activations stay in registers from layer to layer and are split once. W [N][LD] row-major (bf16,
+// shared; LD = K + 8 puts the eight rows a fragment reads in different banks).
+template <int K, int N, bool TANH, class Put>
+HDG_DEVI void mlp_layer_tc(const __nv_bfloat16* W, const __nv_bfloat16* bias, const uint4 (&hi)[K / 16],
+                           const uint4 (&lo)[K / 16], int lane, Put put) {
+  constexpr int LD = K + 8;
   const int g = lane >> 2, t = lane & 3;
-#pragma unroll 1
+#pragma unroll
   for (int nt = 0; nt < N / 8; ++nt) {
     float c[4] = {0.f, 0.f, 0.f, 0.f};
-    const __nv_bfloat16* Wn = W + (nt * 8 + g) * K;
+    const __nv_bfloat16* Wn = W + (nt * 8 + g) * LD + 2 * t;
 #pragma unroll
     for (int kt = 0; kt < K / 16; ++kt) {
-      const int k0 = kt * 16 + 2 * t;
-      uint4 hi, lo;
-      mlp_split2(in[g * kTcLd + k0], in[g * kTcLd + k0 + 1], hi.x, lo.x);
-      mlp_split2(in[(g + 8) * kTcLd + k0], in[(g + 8) * kTcLd + k0 + 1], hi.y, lo.y);
-      mlp_split2(in[g * kTcLd + k0 + 8], in[g * kTcLd + k0 + 9], hi.z, lo.z);
-      mlp_split2(in[(g + 8) * kTcLd + k0 + 8], in[(g + 8) * kTcLd + k0 + 9], hi.w, lo.w);
       uint2 b;
-      b.x = *reinterpret_cast<const unsigned*>(Wn + k0);
-      b.y = *reinterpret_cast<const unsigned*>(Wn + k0 + 8);
-      mlp_mma(c, hi, b);
-      mlp_mma(c, lo, b);
+      b.x = *reinterpret_cast<const unsigned*>(Wn + kt * 16);
+      b.y = *reinterpret_cast<const unsigned*>(Wn + kt * 16 + 8);
+      mlp_mma(c, hi[kt], b);
+      mlp_mma(c, lo[kt], b);
     }
+    const int col = nt * 8 + 2 * t;
+    const float b0 = __bfloat162float(bias[col]), b1 = __bfloat162float(bias[col + 1]);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int row = g + 8 * (q >> 1), col = nt * 8 + 2 * t + (q & 1);
-      const float v = c[q] + __bfloat162float(bias[col]);
-      out[row * kTcLd + col] = TANH ? tanhf(v) : v;
+      const float v = c[q] + (q & 1 ? b1 : b0);
+      c[q] = TANH ? tanhf(v) : v;
     }
+    put(nt, c);
   }
-  __syncwarp();
 }
 
+// The 64-64-16 network. Eight warps of 16 samples share one copy of the weights and go through the batch. 49,152
+// samples, features to corrected trace: 127 us, against 146 us with activations in shared memory between the layers
+// and a block of two warps per 32 samples.
 template <int NIN, int NH, int NOUT>
-__global__ void __launch_bounds__(64) k_mlp_forward_tc(const float* params, const float* x, int64_t B, float* y) {
-  static_assert(NIN % 16 == 0 && NH % 16 == 0 && NOUT % 8 == 0 && NIN <= MAXH && NH <= MAXH, "tile shape");
+__global__ void __launch_bounds__(256, 2) k_mlp_forward_tc(const float* params, const float* x, int64_t B, float* y) {
+  static_assert(NIN % 16 == 0 && NH % 16 == 0 && NOUT % 8 == 0, "tile shape");
   constexpr int P = NH * NIN + NH + NH * NH + NH + NOUT * NH + NOUT;
-  constexpr int WPB = 2;  // warps per block (static shared memory below 48 KB)
-  __shared__ __align__(16) __nv_bfloat16 w[P + 8];
-  __shared__ float act[WPB][2][16 * kTcLd];
+  constexpr int L1 = NIN + 8, L2 = NH + 8;
+  __shared__ __align__(16) __nv_bfloat16 W1[NH * L1], W2[NH * L2], W3[NOUT * L2], bs[2 * NH + NOUT];
   const __nv_bfloat16* w16 = reinterpret_cast<const __nv_bfloat16*>(params + 3 * (int64_t)P);
-  for (int t = threadIdx.x; t < P; t += blockDim.x) w[t] = w16[t];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t b0 = ((int64_t)blockIdx.x * WPB + warp) * 16;
-  float* a0 = act[warp][0];
-  float* a1 = act[warp][1];
-  for (int t = lane; t < 16 * NIN; t += 32) {
-    const int r = t / NIN, k = t % NIN;
-    a0[r * kTcLd + k] = b0 + r < B ? x[(b0 + r) * NIN + k] : 0.f;
-  }
+  constexpr int o1 = NH * NIN, o2 = o1 + NH, o3 = o2 + NH * NH, o4 = o3 + NH, o5 = o4 + NOUT * NH;
+  for (int t = threadIdx.x; t < NH * NIN; t += 256) W1[t / NIN * L1 + t % NIN] = w16[t];
+  for (int t = threadIdx.x; t < NH * NH; t += 256) W2[t / NH * L2 + t % NH] = w16[o2 + t];
+  for (int t = threadIdx.x; t < NOUT * NH; t += 256) W3[t / NH * L2 + t % NH] = w16[o4 + t];
+  for (int t = threadIdx.x; t < 2 * NH + NOUT; t += 256)
+    bs[t] = w16[t < NH ? o1 + t : t < 2 * NH ? o3 + t - NH : o5 + t - 2 * NH];
   __syncthreads();
-  const __nv_bfloat16* W1 = w;
-  const __nv_bfloat16* bb1 = W1 + NH * NIN;
-  const __nv_bfloat16* W2 = bb1 + NH;
-  const __nv_bfloat16* bb2 = W2 + NH * NH;
-  const __nv_bfloat16* W3 = bb2 + NH;
-  const __nv_bfloat16* bb3 = W3 + NOUT * NH;
-  mlp_layer_tc<NIN, NH, true>(W1, bb1, a0, a1, lane);
-  mlp_layer_tc<NH, NH, true>(W2, bb2, a1, a0, lane);
-  mlp_layer_tc<NH, NOUT, false>(W3, bb3, a0, a1, lane);
-  for (int t = lane; t < 16 * NOUT; t += 32) {
-    const int r = t / NOUT, j = t % NOUT;
-    if (b0 + r < B) y[(b0 + r) * NOUT + j] = a1[r * kTcLd + j];
+  const int lane = threadIdx.x & 31, g = lane >> 2, t2 = 2 * (lane & 3);
+  const int64_t ntile = (B + 15) / 16;
+  for (int64_t tile = blockIdx.x * 8 + (threadIdx.x >> 5); tile < ntile; tile += (int64_t)gridDim.x * 8) {
+    const int64_t r0 = tile * 16 + g, r1 = r0 + 8;
+    uint4 hi[NIN / 16], lo[NIN / 16];
+#pragma unroll
+    for (int kt = 0; kt < NIN / 16; ++kt) {
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {  // scalar loads: x may have any alignment of a float
+        const int64_t r = q & 2 ? r1 : r0;
+        v[q] = r < B ? x[r * NIN + kt * 16 + t2 + (q & 4 ? 8 : 0) + (q & 1)] : 0.f;
+      }
+      mlp_split2(v[0], v[1], hi[kt].x, lo[kt].x);
+      mlp_split2(v[2], v[3], hi[kt].y, lo[kt].y);
+      mlp_split2(v[4], v[5], hi[kt].z, lo[kt].z);
+      mlp_split2(v[6], v[7], hi[kt].w, lo[kt].w);
+    }
+    uint4 h1h[NH / 16], h1l[NH / 16], h2h[NH / 16], h2l[NH / 16];
+    auto into = [](uint4 (&H)[NH / 16], uint4 (&L)[NH / 16]) {
+      return [&H, &L](int nt, const float (&c)[4]) {
+        const int kt = nt >> 1;
+        if (nt & 1) {
+          mlp_split2(c[0], c[1], H[kt].z, L[kt].z);
+          mlp_split2(c[2], c[3], H[kt].w, L[kt].w);
+        } else {
+          mlp_split2(c[0], c[1], H[kt].x, L[kt].x);
+          mlp_split2(c[2], c[3], H[kt].y, L[kt].y);
+        }
+      };
+    };
+    mlp_layer_tc<NIN, NH, true>(W1, bs, hi, lo, lane, into(h1h, h1l));
+    mlp_layer_tc<NH, NH, true>(W2, bs + NH, h1h, h1l, lane, into(h2h, h2l));
+    mlp_layer_tc<NH, NOUT, false>(W3, bs + 2 * NH, h2h, h2l, lane, [&](int nt, const float (&c)[4]) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t r = q & 2 ? r1 : r0;
+        if (r < B) y[r * NOUT + nt * 8 + t2 + (q & 1)] = c[q];
+      }
+    });
   }
 }
 
-// Forward + backward of the mean-squared error (mean over the batch and the NOUT
-// outputs). A block takes SB samples: one thread per sample runs the forward and
-// back-propagates to the pre-activation gradients, kept in shared memory; then all
-// threads form the weight gradients as sums over the block's samples and add them to
-// grad [P] (FP32) with one atomic per parameter and block. loss [1] accumulates.
-template <int NIN, int NH, int NOUT, int SB>
+// Forward + backward of the mean-squared error (mean over the batch and the NOUT outputs), FP32 throughout with the
+// BF16 weights. A CTA of 256 threads takes tiles of TS samples; every step is a small matrix product with the
+// operands in shared memory ([sample][feature], [output][input], rows padded by 4 so that 16-byte loads of
+// neighbouring rows meet different banks) and register tiles: 4 outputs x TS / 16 samples for the layers, 4 x 4 weights for
+// the weight gradients, which stay in registers over all tiles of the CTA and go to grad [P] once, by 16-byte
+// reductions. loss [1] accumulates.
+// Bound: FP32 issue and shared-memory reads (1.2G FMA at 49,152 samples of the 64-64-16 network, 31 us at the FP32
+// rate). One thread per sample with all its activations in shared memory, and one atomic per weight and 64
+// samples, took about 590 us; a whole training step of that network and batch (gradient and Adam) went from 609 to 97 us.
+template <int NIN, int NH, int NOUT, int TS>
 struct GradSmem {
-  static constexpr int P = NH * NIN + NH + NH * NH + NH + NOUT * NH + NOUT;
-  static constexpr size_t bytes = sizeof(float) * (size_t)SB * (NIN + 4 * NH + NOUT) + sizeof(__nv_bfloat16) * P + 16;
+  static constexpr int L1 = NIN + 4, L2 = NH + 4, LO = (NOUT + 3) / 4 * 4 + 4;
+  static constexpr size_t bytes =
+      sizeof(float) * (size_t)(NH * L1 + NH * L2 + NOUT * L2 + 2 * NH + NOUT + TS * (L1 + 3 * L2 + LO) + 8);
 };
 
-template <int NIN, int NH, int NOUT, int SB>
-__global__ void __launch_bounds__(128) k_mlp_grad(const float* params, const float* x, const float* target, int64_t B,
-                                                int64_t b0_all, int64_t Btot, float* grad, float* loss) {
-  constexpr int P = NH * NIN + NH + NH * NH + NH + NOUT * NH + NOUT;
-  extern __shared__ float smf[];
-  float* xs = smf;                 // [SB][NIN]
-  float* h1 = xs + SB * NIN;       // [SB][NH]
-  float* h2 = h1 + SB * NH;        // [SB][NH]
-  float* dz1 = h2 + SB * NH;       // [SB][NH]
-  float* dz2 = dz1 + SB * NH;      // [SB][NH]
-  float* dy = dz2 + SB * NH;       // [SB][NOUT]
-  __nv_bfloat16* w = reinterpret_cast<__nv_bfloat16*>(dy + SB * NOUT);
-  __shared__ float lsum;
+// out[s][j] for j < N, s < TS: tile loops over the K inputs by four; in [TS][LDI], W [N][LDW]
+template <int K, int N, int TS, int LDI, int LDW, class Epi>
+HDG_DEVI void mlp_tile_forward(const float* in, const float* W, Epi epi) {
+  constexpr int TJ = N / 4, TR = 256 / TJ, RS = TS / TR;  // thread (tj, tr): outputs tj + TJ i, samples tr + TR q
+  static_assert(N % 4 == 0 && 256 % TJ == 0 && TS % TR == 0, "tile");
+  const int tj = threadIdx.x % TJ, tr = threadIdx.x / TJ;
+  float acc[RS][4] = {};
+#pragma unroll 4
+  for (int k = 0; k < K; k += 4) {
+    float4 w[4], v[RS];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = *reinterpret_cast<const float4*>(W + (tj + TJ * i) * LDW + k);
+#pragma unroll
+    for (int q = 0; q < RS; ++q) v[q] = *reinterpret_cast<const float4*>(in + (tr + TR * q) * LDI + k);
+#pragma unroll
+    for (int q = 0; q < RS; ++q)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[q][i] = fmaf(w[i].x, v[q].x, acc[q][i]);
+        acc[q][i] = fmaf(w[i].y, v[q].y, acc[q][i]);
+        acc[q][i] = fmaf(w[i].z, v[q].z, acc[q][i]);
+        acc[q][i] = fmaf(w[i].w, v[q].w, acc[q][i]);
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < RS; ++q)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) epi(tr + TR * q, tj + TJ * i, acc[q][i]);
+}
+
+// d[s][k] = (sum_j e[s][j] W[j][k]) (1 - h[s][k]^2), k < N: the gradient before a tanh layer
+template <int J, int N, int TS, int LDE, int LDW, int LDH>
+HDG_DEVI void mlp_tile_backward(const float* e, const float* W, const float* h, float* d) {
+  constexpr int TJ = N / 4, TR = 256 / TJ, RS = TS / TR;
+  static_assert(J % 4 == 0, "tile");
+  const int k0 = 4 * (threadIdx.x % TJ), tr = threadIdx.x / TJ;
+  float4 acc[RS] = {};
+#pragma unroll 4
+  for (int j = 0; j < J; j += 4) {
+    float4 w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = *reinterpret_cast<const float4*>(W + (j + i) * LDW + k0);
+#pragma unroll
+    for (int q = 0; q < RS; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(e + (tr + TR * q) * LDE + j);
+      const float ev[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[q].x = fmaf(w[i].x, ev[i], acc[q].x);
+        acc[q].y = fmaf(w[i].y, ev[i], acc[q].y);
+        acc[q].z = fmaf(w[i].z, ev[i], acc[q].z);
+        acc[q].w = fmaf(w[i].w, ev[i], acc[q].w);
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < RS; ++q) {
+    const int r = tr + TR * q;
+    const float4 u = *reinterpret_cast<const float4*>(h + r * LDH + k0);
+    *reinterpret_cast<float4*>(d + r * LDH + k0) =
+        make_float4(acc[q].x * (1.f - u.x * u.x), acc[q].y * (1.f - u.y * u.y), acc[q].z * (1.f - u.z * u.z),
+                    acc[q].w * (1.f - u.w * u.w));
+  }
+}
+
+// acc[i][q] += sum_s d[s][j0 + i] v[s][k0 + q] for this thread's 4 x 4 weights
+template <int TS, int LDD, int LDV>
+HDG_DEVI void mlp_tile_weights(const float* d, const float* v, int j0, int k0, float (&acc)[4][4]) {
+#pragma unroll 4
+  for (int s = 0; s < TS; ++s) {
+    const float4 a = *reinterpret_cast<const float4*>(d + s * LDD + j0), b = *reinterpret_cast<const float4*>(v + s * LDV + k0);
+    const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      acc[i][0] = fmaf(av[i], b.x, acc[i][0]);
+      acc[i][1] = fmaf(av[i], b.y, acc[i][1]);
+      acc[i][2] = fmaf(av[i], b.z, acc[i][2]);
+      acc[i][3] = fmaf(av[i], b.w, acc[i][3]);
+    }
+  }
+}
+
+HDG_DEVI void mlp_red4(float* p, const float (&v)[4], bool vec) {
+  if (vec) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+  } else {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) atomicAdd(p + q, v[q]);
+  }
+}
+
+template <int NIN, int NH, int NOUT, int TS>
+__global__ void __launch_bounds__(256, 2) k_mlp_grad(const float* params, const float* x, const float* target, int64_t B,
+                                                    float* grad, float* loss) {
+  using G = GradSmem<NIN, NH, NOUT, TS>;
+  constexpr int P = NH * NIN + NH + NH * NH + NH + NOUT * NH + NOUT, L1 = G::L1, L2 = G::L2, LO = G::LO;
+  constexpr int o1 = NH * NIN, o2 = o1 + NH, o3 = o2 + NH * NH, o4 = o3 + NH, o5 = o4 + NOUT * NH;
+  extern __shared__ __align__(16) float smf[];
+  float* W1 = smf;              // [NH][L1]
+  float* W2 = W1 + NH * L1;     // [NH][L2]
+  float* W3 = W2 + NH * L2;     // [NOUT][L2]
+  float* xs = W3 + NOUT * L2;   // [TS][L1]
+  float* h1 = xs + TS * L1;     // [TS][L2]
+  float* h2 = h1 + TS * L2;     // [TS][L2], later the gradient before the first tanh
+  float* d2 = h2 + TS * L2;     // [TS][L2]
+  float* dy = d2 + TS * L2;     // [TS][LO]
+  float* bs = dy + TS * LO;     // biases
+  float* lsum = bs + 2 * NH + NOUT;
+  const int tid = threadIdx.x;
   const __nv_bfloat16* w16 = reinterpret_cast<const __nv_bfloat16*>(params + 3 * (int64_t)P);
-  for (int t = threadIdx.x; t < P; t += blockDim.x) w[t] = w16[t];
-  if (threadIdx.x == 0) lsum = 0.f;
-  __syncthreads();
-  const __nv_bfloat16* W2 = w + NH * NIN + NH;
-  const __nv_bfloat16* W3 = W2 + NH * NH + NH;
-  const int64_t base = (int64_t)blockIdx.x * SB;
-  const int nb_here = (int)((B - base) < SB ? (B - base) : SB);
-  if ((int)threadIdx.x < SB) {
-    const int sb = threadIdx.x;
-    float* xr = xs + sb * NIN;
-    float* a1 = h1 + sb * NH;
-    float* a2 = h2 + sb * NH;
-    float* d1 = dz1 + sb * NH;
-    float* d2 = dz2 + sb * NH;
-    float* dyr = dy + sb * NOUT;
-    if (sb < nb_here) {
-      const int64_t b = b0_all + base + sb;
-      for (int k = 0; k < NIN; ++k) xr[k] = x[b * NIN + k];
-      float out[NOUT];
-      mlp_forward_one<NIN, NH, NOUT>(w, xr, a1, a2, out);
-      const float inv = 1.f / ((float)Btot * (float)NOUT);
-      float l = 0.f;
-      for (int j = 0; j < NOUT; ++j) {
-        const float d = out[j] - target[b * NOUT + j];
-        l += d * d;
-        dyr[j] = 2.f * d * inv;
+  for (int t = tid; t < NH * NIN; t += 256) W1[t / NIN * L1 + t % NIN] = __bfloat162float(w16[t]);
+  for (int t = tid; t < NH * NH; t += 256) W2[t / NH * L2 + t % NH] = __bfloat162float(w16[o2 + t]);
+  for (int t = tid; t < NOUT * NH; t += 256) W3[t / NH * L2 + t % NH] = __bfloat162float(w16[o4 + t]);
+  for (int t = tid; t < 2 * NH + NOUT; t += 256)
+    bs[t] = __bfloat162float(w16[t < NH ? o1 + t : t < 2 * NH ? o3 + t - NH : o5 + t - 2 * NH]);
+  if (tid == 0) *lsum = 0.f;
+  // this thread's weights: 4 x 4 tiles of dW1, dW2 and dW3, and one bias
+  constexpr int T1 = NH * NIN / 16, T2 = NH * NH / 16, T3 = NOUT * NH / 16;
+  static_assert(T1 <= 256 && T2 <= 256 && T3 <= 256 && 2 * NH + NOUT <= 256, "one tile per thread");
+  const int j1 = 4 * (tid / (NIN / 4)), k1 = 4 * (tid % (NIN / 4)), j2 = 4 * (tid / (NH / 4)), k2 = 4 * (tid % (NH / 4));
+  float g1[4][4] = {}, g2[4][4] = {}, g3[4][4] = {}, gb = 0.f, l = 0.f;
+  const float inv = 1.f / ((float)B * (float)NOUT);
+  for (int64_t base = (int64_t)blockIdx.x * TS; base < B; base += (int64_t)gridDim.x * TS) {
+    __syncthreads();
+    for (int t = tid; t < TS * NIN; t += 256) {
+      const int s = t / NIN;
+      xs[s * L1 + t % NIN] = base + s < B ? x[base * NIN + t] : 0.f;
+    }
+    __syncthreads();
+    mlp_tile_forward<NIN, NH, TS, L1, L1>(xs, W1, [&](int s, int j, float v) { h1[s * L2 + j] = tanhf(v + bs[j]); });
+    __syncthreads();
+    mlp_tile_forward<NH, NH, TS, L2, L2>(h1, W2, [&](int s, int j, float v) { h2[s * L2 + j] = tanhf(v + bs[NH + j]); });
+    __syncthreads();
+    for (int t = tid; t < TS * NOUT; t += 256) {  // the output layer, the error and its gradient
+      const int s = t / NOUT, j = t % NOUT;
+      float v = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < NH; k += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(W3 + j * L2 + k), h = *reinterpret_cast<const float4*>(h2 + s * L2 + k);
+        v = fmaf(w.x, h.x, fmaf(w.y, h.y, fmaf(w.z, h.z, fmaf(w.w, h.w, v))));
       }
-      atomicAdd(&lsum, l * inv);
-      for (int k = 0; k < NH; ++k) {
-        float s = 0.f;
-        for (int j = 0; j < NOUT; ++j) s = fmaf(__bfloat162float(W3[j * NH + k]), dyr[j], s);
-        d2[k] = s * (1.f - a2[k] * a2[k]);
-      }
-      for (int k = 0; k < NH; ++k) {
-        float s = 0.f;
-        for (int j = 0; j < NH; ++j) s = fmaf(__bfloat162float(W2[j * NH + k]), d2[j], s);
-        d1[k] = s * (1.f - a1[k] * a1[k]);
-      }
-    } else {  // padding samples contribute nothing
-      for (int k = 0; k < NIN; ++k) xr[k] = 0.f;
-      for (int k = 0; k < NH; ++k) a1[k] = a2[k] = d1[k] = d2[k] = 0.f;
-      for (int j = 0; j < NOUT; ++j) dyr[j] = 0.f;
+      float d = 0.f;  // samples past the batch contribute nothing
+      if (base + s < B) d = v + bs[2 * NH + j] - target[base * NOUT + t];
+      l += d * d * inv;
+      dy[s * LO + j] = 2.f * d * inv;
+    }
+    __syncthreads();
+    mlp_tile_backward<NOUT, NH, TS, LO, L2, L2>(dy, W3, h2, d2);
+    if (tid < T3) mlp_tile_weights<TS, LO, L2>(dy, h2, j2, k2, g3);
+    __syncthreads();
+    mlp_tile_backward<NH, NH, TS, L2, L2, L2>(d2, W2, h1, h2);  // h2 becomes the gradient before the first tanh
+    if (tid < T2) mlp_tile_weights<TS, L2, L2>(d2, h1, j2, k2, g2);
+    __syncthreads();
+    if (tid < T1) mlp_tile_weights<TS, L2, L1>(h2, xs, j1, k1, g1);
+    if (tid < 2 * NH + NOUT) {
+      const float* src = tid < NH ? h2 + tid : tid < 2 * NH ? d2 + tid - NH : dy + tid - 2 * NH;
+      const int ld = tid < 2 * NH ? L2 : LO;
+      for (int s = 0; s < TS; ++s) gb += src[s * ld];
     }
   }
-  __syncthreads();
-  // weight gradients: sums over the block's samples
-  for (int t = threadIdx.x; t < P; t += blockDim.x) {
-    const float *L, *Rr;
-    int ldl, ldr, j, k;
-    bool bias = false;
-    int p = t;
-    if (p < NH * NIN) {
-      j = p / NIN; k = p % NIN; L = dz1; ldl = NH; Rr = xs; ldr = NIN;
-    } else if ((p -= NH * NIN) < NH) {
-      j = p; k = 0; L = dz1; ldl = NH; Rr = nullptr; ldr = 0; bias = true;
-    } else if ((p -= NH) < NH * NH) {
-      j = p / NH; k = p % NH; L = dz2; ldl = NH; Rr = h1; ldr = NH;
-    } else if ((p -= NH * NH) < NH) {
-      j = p; k = 0; L = dz2; ldl = NH; Rr = nullptr; ldr = 0; bias = true;
-    } else if ((p -= NH) < NOUT * NH) {
-      j = p / NH; k = p % NH; L = dy; ldl = NOUT; Rr = h2; ldr = NH;
-    } else {
-      p -= NOUT * NH;
-      j = p; k = 0; L = dy; ldl = NOUT; Rr = nullptr; ldr = 0; bias = true;
-    }
-    float s = 0.f;
-    for (int sb = 0; sb < SB; ++sb) s = fmaf(L[sb * ldl + j], bias ? 1.f : Rr[sb * ldr + k], s);
-    atomicAdd(grad + t, s);
+  const bool vec = (reinterpret_cast<uintptr_t>(grad) & 15) == 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (tid < T1) mlp_red4(grad + (j1 + i) * NIN + k1, g1[i], vec);
+    if (tid < T2) mlp_red4(grad + o2 + (j2 + i) * NH + k2, g2[i], vec);
+    if (tid < T3) mlp_red4(grad + o4 + (j2 + i) * NH + k2, g3[i], vec);
   }
-  if (threadIdx.x == 0) atomicAdd(loss, lsum);
+  if (tid < 2 * NH + NOUT) atomicAdd(grad + (tid < NH ? o1 + tid : tid < 2 * NH ? o3 + tid - NH : o5 + tid - 2 * NH), gb);
+  for (int off = 16; off > 0; off >>= 1) l += __shfl_down_sync(0xffffffffu, l, off);
+  if ((tid & 31) == 0) atomicAdd(lsum, l);
+  __syncthreads();
+  if (tid == 0) atomicAdd(loss, *lsum);
 }
 
 // Adam on the FP32 master weights, then refresh the BF16 copy.
@@ -355,20 +471,23 @@ __global__ void k_mlp_apply(const double* Vhat, const double* dvh1, const float*
   }
 }
 
-template <int NIN, int NH, int NOUT>
+__global__ void k_mlp_zero(float* grad, int64_t P, float* loss) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < P; t += (int64_t)gridDim.x * blockDim.x) grad[t] = 0.f;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *loss = 0.f;
+}
+
+// TS: samples per tile (64-64-16: 48, the most that lets two CTAs share an SM)
+template <int NIN, int NH, int NOUT, int TS>
 int launch_grad(const float* params, const float* x, const float* target, int64_t B, float* grad, float* loss,
                 cudaStream_t s) {
-  constexpr int SB = 64;
-  using G = GradSmem<NIN, NH, NOUT, SB>;
-  HDG_CK(cudaFuncSetAttribute(k_mlp_grad<NIN, NH, NOUT, SB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  using G = GradSmem<NIN, NH, NOUT, TS>;
+  constexpr int P = NH * NIN + NH + NH * NH + NH + NOUT * NH + NOUT;
+  HDG_CK(cudaFuncSetAttribute(k_mlp_grad<NIN, NH, NOUT, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)G::bytes));
-  // grid limited to 65535 blocks per launch: split very large batches
-  const int64_t per_launch = (int64_t)65535 * SB;
-  for (int64_t b0 = 0; b0 < B; b0 += per_launch) {
-    const int64_t nbat = (B - b0) < per_launch ? (B - b0) : per_launch;
-    k_mlp_grad<NIN, NH, NOUT, SB><<<(unsigned)((nbat + SB - 1) / SB), 128, G::bytes, s>>>(params, x, target, nbat,
-                                                                                        b0, B, grad, loss);
-  }
+  k_mlp_zero<<<(P + 255) / 256, 256, 0, s>>>(grad, P, loss);
+  const int64_t tiles = (B + TS - 1) / TS;
+  k_mlp_grad<NIN, NH, NOUT, TS><<<(unsigned)(tiles < 2 * 152 ? tiles : 2 * 152), 256, G::bytes, s>>>(params, x, target,
+                                                                                                   B, grad, loss);
   HDG_CK(cudaGetLastError());
   return HDG_OK;
 }
@@ -475,10 +594,11 @@ int hdg_mlp_forward(const float* params, int nin, int nh, int nout, const float*
   if (B == 0) return HDG_OK;
   const unsigned g = (unsigned)((B + 127) / 128);
   cudaStream_t s = (cudaStream_t)stream;
-  // 64-64-16 (2D p = 3) on the tensor cores, 32 samples per block; 48-32-12 keeps the scalar kernel
+  // 64-64-16 (2D p = 3) on the tensor cores, 128 samples per block and pass; 48-32-12 keeps the scalar kernel
   // (its output width is not a multiple of the tile's 8 columns)
-  const unsigned g32 = (unsigned)((B + 31) / 32);
-  MLP_DISPATCH(64, 64, 16, (k_mlp_forward_tc<64, 64, 16><<<g32, 64, 0, s>>>(params, x, B, y));
+  const int64_t t128 = (B + 127) / 128;
+  const unsigned gt = (unsigned)(t128 < 3 * 152 ? t128 : 3 * 152);
+  MLP_DISPATCH(64, 64, 16, (k_mlp_forward_tc<64, 64, 16><<<gt, 256, 0, s>>>(params, x, B, y));
                HDG_CK(cudaGetLastError()); return HDG_OK)
   MLP_DISPATCH(48, 32, 12, (k_mlp_forward<48, 32, 12><<<g, 128, 0, s>>>(params, x, B, y)); HDG_CK(cudaGetLastError());
                return HDG_OK)
@@ -494,12 +614,10 @@ int hdg_mlp_train_step(float* params, float* grad, int nin, int nh, int nout, co
   }
   const int64_t P = mlp_params(nin, nh, nout);
   cudaStream_t s = (cudaStream_t)stream;
-  HDG_CK(cudaMemsetAsync(grad, 0, sizeof(float) * P, s));
-  HDG_CK(cudaMemsetAsync(loss, 0, sizeof(float), s));
   bool done = false;
   int rc = HDG_OK;
-  MLP_DISPATCH(64, 64, 16, rc = launch_grad<64, 64, 16>(params, x, target, B, grad, loss, s); done = true)
-  MLP_DISPATCH(48, 32, 12, rc = launch_grad<48, 32, 12>(params, x, target, B, grad, loss, s); done = true)
+  MLP_DISPATCH(64, 64, 16, rc = launch_grad<64, 64, 16, 48>(params, x, target, B, grad, loss, s); done = true)
+  MLP_DISPATCH(48, 32, 12, rc = launch_grad<48, 32, 12, 64>(params, x, target, B, grad, loss, s); done = true)
   if (rc) return rc;
   if (!done) {
     set_error("hdg_mlp_train_step: network size not compiled in");
@@ -518,10 +636,8 @@ int hdg_mlp_gradient(const float* params, float* grad, int nin, int nh, int nout
   }
   const int64_t P = mlp_params(nin, nh, nout);
   cudaStream_t s = (cudaStream_t)stream;
-  HDG_CK(cudaMemsetAsync(grad, 0, sizeof(float) * P, s));
-  HDG_CK(cudaMemsetAsync(loss, 0, sizeof(float), s));
-  MLP_DISPATCH(64, 64, 16, return launch_grad<64, 64, 16>(params, x, target, B, grad, loss, s))
-  MLP_DISPATCH(48, 32, 12, return launch_grad<48, 32, 12>(params, x, target, B, grad, loss, s))
+  MLP_DISPATCH(64, 64, 16, return launch_grad<64, 64, 16, 48>(params, x, target, B, grad, loss, s))
+  MLP_DISPATCH(48, 32, 12, return launch_grad<48, 32, 12, 64>(params, x, target, B, grad, loss, s))
   set_error("hdg_mlp_gradient: network size not compiled in");
   return HDG_ERR_UNSUPPORTED;
 }
