@@ -48,6 +48,50 @@ __device__ double block_sum(double v) {
   return s;
 }
 
+// Rows [0, nr) of a row-major matrix with nc columns times xs (shared memory), FP64; done(row, value) per row by one lane.
+// GB300's FP64 pipe (two FMA per clock and SM) is as tight as HBM here, so what counts is FP64 instructions
+// per entry: half a warp takes eight rows at a time and folds its eight sums together while it adds them up over
+// its lanes (8 additions for 16 rows, where one sum per warp and row takes 5 for each row).
+// 3D p = 3, 10,368 elements: product 941 us (one row per warp: 1,456), whose FMAs alone take 720 us and whose bytes
+// 490 us; recovery 453 us (784), FMAs 360 us.
+template <class Done>
+HDG_DEVI void rows_times_vector(const double* __restrict__ A, int nr, int nc, const double* xs, Done done) {
+  const int lane = threadIdx.x & 31, hl = lane & 15, half = (threadIdx.x >> 4), nhalf = blockDim.x >> 4;
+  for (int r0 = half * 8; r0 - (half & 1) * 8 < nr; r0 += nhalf * 8) {  // both halves of a warp stay together
+    double s[8] = {};
+    const double* p[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = A + (int64_t)min(r0 + i, nr - 1) * nc;
+    if (r0 < nr)
+#pragma unroll 2
+      for (int c = hl; c < nc; c += 16) {
+        const double x = xs[c];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] += p[i][c] * x;
+      }
+    // lane hl ends with the sum of row r0 + 4 (bit 3) + 2 (bit 2) + (bit 1)
+    const bool b3 = hl & 8, b2 = hl & 4, b1 = hl & 2;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double give = b3 ? s[i] : s[i + 4], keep = b3 ? s[i + 4] : s[i];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const double give = b2 ? s[i] : s[i + 2], keep = b2 ? s[i + 2] : s[i];
+      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+    }
+    const double give = b1 ? s[0] : s[1], keep = b1 ? s[1] : s[0];
+    double v = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    const int row = r0 + (b3 ? 4 : 0) + (b2 ? 2 : 0) + (b1 ? 1 : 0);
+    if (!(hl & 1) && row < nr) done(row, v);
+  }
+}
+
+// threads of a CTA that takes `rows` rows: a warp per 16, at most eight
+inline unsigned row_threads(int rows) { return 32u * (unsigned)std::min(8, (rows + 15) / 16); }
+
 // ---------------------------------------------------------------- element data
 template <int D>
 __global__ void k_prim_to_entropy(const double* prim, int64_t n, double gamma, double* v) {
@@ -221,9 +265,8 @@ __global__ void k_node_gather(const int* ptr, const int* occ, int64_t nnode, int
   }
 }
 
-// w_e = S_e x_e in FP64, one warp per row, x_e gathered into shared memory. On GB300 this is
-// bound by the FP64 pipe (one FMA per 8-byte entry), not by HBM: the GMRES iterations use the
-// double-float copy of S (k_elem_matvec_df) and keep this one for the residuals.
+// w_e = S_e x_e in FP64, x_e gathered into shared memory. The GMRES iterations use the double-float copy of S
+// (k_elem_matvec_df) and keep this one for the residuals.
 __global__ void k_elem_matvec(const double* S, const double* x, const int* tgidx, int NT, int M, double* w, const int* skip) {
   if (skip && *skip) return;  // a finished Krylov cycle: nothing to do
   extern __shared__ double xs[];
@@ -234,14 +277,7 @@ __global__ void k_elem_matvec(const double* S, const double* x, const int* tgidx
     xs[t] = x[(int64_t)tgidx[e * nfc + fc] * M + i];
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const double* Se = S + e * (int64_t)NT * NT;
-  for (int r = wid; r < NT; r += nw) {
-    double s = 0.0;
-    for (int c = lane; c < NT; c += 32) s += Se[(int64_t)r * NT + c] * xs[c];
-    s = warp_sum(s);
-    if (lane == 0) w[e * NT + r] = s;
-  }
+  rows_times_vector(S + e * (int64_t)NT * NT, NT, NT, xs, [&](int r, double v) { w[e * NT + r] = v; });
 }
 
 // The double-float copy of S: entry i = hi + lo (hi = S rounded to FP32, lo = the rest rounded),
@@ -262,15 +298,9 @@ __global__ void k_recover(const double* recov, const double* dvh, const int* tgi
     xs[t] = dvh[(int64_t)tgidx[e * nfc + fc] * M + i];
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const double* X = recov + e * (int64_t)(NV * NT + NV);
   const double* y = X + (int64_t)NV * NT;
-  for (int r = wid; r < NV; r += nw) {
-    double s = 0.0;
-    for (int c = lane; c < NT; c += 32) s += X[(int64_t)r * NT + c] * xs[c];
-    s = warp_sum(s);
-    if (lane == 0) dV[e * NV + r] = -y[r] - s;
-  }
+  rows_times_vector(X, NV, NT, xs, [&](int r, double v) { dV[e * NV + r] = -y[r] - v; });
 }
 
 __global__ void k_sumsq_elem_rows(const double* R, int64_t E, int stride, int n, double* out) {
@@ -800,8 +830,8 @@ int launch_trace_matvec(hdg_ctx* ctx, const double* S, const double* x, double* 
     if (int rc = pm_elem_matvec(ctx, S, x, work, s, skip)) return rc;
     return pm_gather(ctx, work, 1.0, y, s, skip);
   }
-  k_elem_matvec<<<(unsigned)ctx->E, 256, sizeof(double) * ctx->NT, s>>>(S, x, ctx->d_tgidx, ctx->NT, ctx->M, work,
-                                                                        skip);
+  k_elem_matvec<<<(unsigned)ctx->E, row_threads(ctx->NT), sizeof(double) * ctx->NT, s>>>(S, x, ctx->d_tgidx, ctx->NT,
+                                                                                      ctx->M, work, skip);
   return launch_gather(ctx, work, y, s, skip);
 }
 
@@ -844,8 +874,8 @@ static int launch_trace_matvec_df(hdg_ctx* ctx, const df2* Sdf, const double* x,
 
 int launch_recover(hdg_ctx* ctx, const double* recov, const double* dVhat, double* dV, cudaStream_t s) {
   if (ctx->pm) return pm_recover(ctx, recov, dVhat, dV, s);
-  k_recover<<<(unsigned)ctx->E, 256, sizeof(double) * ctx->NT, s>>>(recov, dVhat, ctx->d_tgidx, ctx->NV, ctx->NT,
-                                                                   ctx->M, dV);
+  k_recover<<<(unsigned)ctx->E, row_threads(ctx->NV), sizeof(double) * ctx->NT, s>>>(recov, dVhat, ctx->d_tgidx, ctx->NV,
+                                                                                  ctx->NT, ctx->M, dV);
   HDG_CK(cudaGetLastError());
   return HDG_OK;
 }
