@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "ctx.hpp"
+#include "dense_lu.cuh"
 #include "dfloat.cuh"
 #include "ptx_async.cuh"
 
@@ -662,82 +663,6 @@ __global__ void k_dense_scatter(const double* S, const int* tgidx, int64_t E, in
     atomicAdd(K + gr * n + gc, S[t]);
   }
 }
-__global__ void k_dense_pivot(double* K, int64_t n, int64_t k, int* piv, int* bad) {
-  __shared__ double bv[1024];
-  __shared__ int64_t bi[1024];
-  double best = -1.0;
-  int64_t idx = k;
-  for (int64_t r = k + threadIdx.x; r < n; r += blockDim.x) {
-    double v = fabs(K[r * n + k]);
-    if (v > best) {
-      best = v;
-      idx = r;
-    }
-  }
-  bv[threadIdx.x] = best;
-  bi[threadIdx.x] = idx;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      double ov = bv[threadIdx.x + s];
-      int64_t oi = bi[threadIdx.x + s];
-      if (ov > bv[threadIdx.x] || (ov == bv[threadIdx.x] && oi < bi[threadIdx.x])) {
-        bv[threadIdx.x] = ov;
-        bi[threadIdx.x] = oi;
-      }
-    }
-    __syncthreads();
-  }
-  const int64_t p = bi[0];
-  if (threadIdx.x == 0) {
-    piv[k] = (int)p;
-    if (!(bv[0] > 0.0)) *bad = 1;
-  }
-  if (p != k)
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-      double t = K[k * n + j];
-      K[k * n + j] = K[p * n + j];
-      K[p * n + j] = t;
-    }
-}
-__global__ void k_dense_scale(double* K, int64_t n, int64_t k) {
-  const double d = K[k * n + k];
-  const double inv = d != 0.0 ? 1.0 / d : 0.0;
-  for (int64_t r = k + 1 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x)
-    K[r * n + k] *= inv;
-}
-__global__ void k_dense_update(double* K, int64_t n, int64_t k) {
-  const int64_t rem = n - k - 1;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < rem * rem; t += (int64_t)gridDim.x * blockDim.x) {
-    int64_t r = k + 1 + t / rem, c = k + 1 + t % rem;
-    K[r * n + c] -= K[r * n + k] * K[k * n + c];
-  }
-}
-// forward / backward substitution in one block
-__global__ void k_dense_solve(const double* K, const int* piv, int64_t n, double* x) {
-  if (threadIdx.x == 0)
-    for (int64_t k = 0; k < n; ++k) {
-      int64_t p = piv[k];
-      if (p != k) {
-        double t = x[k];
-        x[k] = x[p];
-        x[p] = t;
-      }
-    }
-  __syncthreads();
-  for (int64_t k = 0; k < n; ++k) {
-    double xk = x[k];
-    for (int64_t r = k + 1 + threadIdx.x; r < n; r += blockDim.x) x[r] -= K[r * n + k] * xk;
-    __syncthreads();
-  }
-  for (int64_t k = n - 1; k >= 0; --k) {
-    if (threadIdx.x == 0) x[k] /= K[k * n + k];
-    __syncthreads();
-    double xk = x[k];
-    for (int64_t r = threadIdx.x; r < k; r += blockDim.x) x[r] -= K[r * n + k] * xk;
-    __syncthreads();
-  }
-}
 
 }  // namespace
 
@@ -935,7 +860,7 @@ static int dense_solve(hdg_ctx* ctx, const double* S, const double* g, double* d
     ctx->d_dpiv = nullptr;
     ctx->dense_n = 0;
     HDG_CK(cudaMalloc(&ctx->d_dense, sizeof(double) * n * n));
-    HDG_CK(cudaMalloc(&ctx->d_dpiv, sizeof(int) * (n + 1)));
+    HDG_CK(cudaMalloc(&ctx->d_dpiv, sizeof(int) * (n + 1 + n / 32 + 1)));  // pivots, zero-pivot flag, tile flags
     ctx->dense_n = (size_t)n;
     if (ctx->lu_graph_exec) {  // the recorded graph refers to the old buffers
       cudaGraphExecDestroy(ctx->lu_graph_exec);
@@ -954,21 +879,17 @@ static int dense_solve(hdg_ctx* ctx, const double* S, const double* g, double* d
     k_dense_scatter<<<nblocks(ctx->E * (int64_t)ctx->NT * ctx->NT), kThreads, 0, s>>>(S, ctx->d_tgidx, ctx->E,
                                                                                      ctx->NT, ctx->M, n, K);
   }
-  // LU with partial pivoting: 3 launches per pivot, recorded once per context into a CUDA
-  // graph (on a context-owned stream, so the caller's stream may be the legacy default
-  // stream) and replayed on the caller's stream.
+  // LU with partial pivoting (dense_lu.cuh), recorded once per context into a CUDA graph (on a
+  // context-owned stream, so the caller's stream may be the legacy default stream) and replayed on
+  // the caller's stream.
   if (!ctx->lu_graph_exec) {
+    HDG_CK(cudaFuncSetAttribute(k_lu_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_panel_smem(kLuMaxN)));
+    HDG_CK(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kLuMaxN * (int)sizeof(double)));
     cudaStream_t cap = nullptr;
     HDG_CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
     HDG_CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-    for (int64_t k = 0; k < n; ++k) {
-      k_dense_pivot<<<1, 1024, 0, cap>>>(K, n, k, ctx->d_dpiv, bad);
-      if (k + 1 < n) {
-        k_dense_scale<<<nblocks(n - k - 1), kThreads, 0, cap>>>(K, n, k);
-        k_dense_update<<<nblocks((n - k - 1) * (n - k - 1)), kThreads, 0, cap>>>(K, n, k);
-      }
-    }
+    enqueue_lu(K, n, ctx->d_dpiv, bad, ctx->d_dpiv + n + 1, cap);
     cudaError_t ce = cudaStreamEndCapture(cap, &graph);
     cudaStreamDestroy(cap);
     if (ce != cudaSuccess) return cuda_fail(ce, "cudaStreamEndCapture (dense LU)");
@@ -985,7 +906,7 @@ static int dense_solve(hdg_ctx* ctx, const double* S, const double* g, double* d
   }
   rc = launch_trace_rhs(ctx, g, dVhat, s);
   if (rc) return rc;
-  k_dense_solve<<<1, 1024, 0, s>>>(K, ctx->d_dpiv, n, dVhat);
+  k_lu_solve<<<kLuCluster, 256, sizeof(double) * n, s>>>(K, ctx->d_dpiv, n, dVhat);
   HDG_CK(cudaGetLastError());
   int hbad = 0;
   HDG_CK(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1229,7 +1150,7 @@ int trace_solve(hdg_ctx* ctx, const double* S, const double* g, double* dVhat, i
                 int* iters, double* final_res, cudaStream_t s) {
   if (method == HDG_SOLVER_AUTO) method = ctx->ntrace <= 4096 ? HDG_SOLVER_DENSE : HDG_SOLVER_GMRES;
   if (method == HDG_SOLVER_DENSE) {
-    if (ctx->ntrace > 16384) {
+    if (ctx->ntrace > kLuMaxN) {
       set_error("trace_solve: dense solver limited to n_trace <= 16384");
       return HDG_ERR_INVALID_ARG;
     }
