@@ -49,44 +49,66 @@ __device__ double block_sum(double v) {
   return s;
 }
 
-// Rows [0, nr) of a row-major matrix with nc columns times xs (shared memory), FP64; done(row, value) per row by one lane.
-// GB300's FP64 pipe (two FMA per clock and SM) is as tight as HBM here, so what counts is FP64 instructions
+// Accumulators of rows_times_vector: FP64, and double-float (dfloat.cuh: exact products by FMA residuals, two-sums).
+struct RowF64 {
+  using T = double;
+  double v = 0.0;
+  HDG_DEVI void mac(double a, double x) { v += a * x; }
+  HDG_DEVI void fold(const RowF64& give, int m) { v += __shfl_xor_sync(0xffffffffu, give.v, m); }
+  HDG_DEVI double value() const { return v; }
+};
+struct RowDf {
+  using T = df2;
+  dfacc v;
+  HDG_DEVI void mac(const df2& a, const df2& x) { v.mac(a, x); }
+  HDG_DEVI void fold(const RowDf& give, int m) {
+    const float h = __shfl_xor_sync(0xffffffffu, give.v.hi, m), l = __shfl_xor_sync(0xffffffffu, give.v.lo, m);
+    v.add(df2{h, l});
+  }
+  HDG_DEVI double value() const { return v.value(); }
+};
+
+// Rows [0, nr) of a row-major matrix with nc columns times xs (shared memory); done(row, value) per row by one lane.
+// In FP64 GB300's pipe (two FMA per clock and SM) is as tight as HBM, so what counts is FP64 instructions
 // per entry: half a warp takes eight rows at a time and folds its eight sums together while it adds them up over
 // its lanes (8 additions for 16 rows, where one sum per warp and row takes 5 for each row).
 // 3D p = 3, 10,368 elements: product 941 us (one row per warp: 1,456), whose FMAs alone take 720 us and whose bytes
 // 490 us; recovery 453 us (784), FMAs 360 us.
-template <class Done>
-HDG_DEVI void rows_times_vector(const double* __restrict__ A, int nr, int nc, const double* xs, Done done) {
+template <class Acc, class Done>
+HDG_DEVI void rows_times_vector(const typename Acc::T* __restrict__ A, int nr, int nc, const typename Acc::T* xs, Done done) {
   const int lane = threadIdx.x & 31, hl = lane & 15, half = (threadIdx.x >> 4), nhalf = blockDim.x >> 4;
   for (int r0 = half * 8; r0 - (half & 1) * 8 < nr; r0 += nhalf * 8) {  // both halves of a warp stay together
-    double s[8] = {};
-    const double* p[8];
+    Acc s[8];
+    const typename Acc::T* p[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) p[i] = A + (int64_t)min(r0 + i, nr - 1) * nc;
     if (r0 < nr)
 #pragma unroll 2
       for (int c = hl; c < nc; c += 16) {
-        const double x = xs[c];
+        const typename Acc::T x = xs[c];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] += p[i][c] * x;
+        for (int i = 0; i < 8; ++i) s[i].mac(p[i][c], x);
       }
     // lane hl ends with the sum of row r0 + 4 (bit 3) + 2 (bit 2) + (bit 1)
     const bool b3 = hl & 8, b2 = hl & 4, b1 = hl & 2;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const double give = b3 ? s[i] : s[i + 4], keep = b3 ? s[i + 4] : s[i];
-      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+      const Acc give = b3 ? s[i] : s[i + 4];
+      s[i] = b3 ? s[i + 4] : s[i];
+      s[i].fold(give, 8);
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const double give = b2 ? s[i] : s[i + 2], keep = b2 ? s[i + 2] : s[i];
-      s[i] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+      const Acc give = b2 ? s[i] : s[i + 2];
+      s[i] = b2 ? s[i + 2] : s[i];
+      s[i].fold(give, 4);
     }
-    const double give = b1 ? s[0] : s[1], keep = b1 ? s[1] : s[0];
-    double v = keep + __shfl_xor_sync(0xffffffffu, give, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    const Acc give = b1 ? s[0] : s[1];
+    Acc v = b1 ? s[1] : s[0];
+    v.fold(give, 2);
+    v.fold(Acc(v), 1);
     const int row = r0 + (b3 ? 4 : 0) + (b2 ? 2 : 0) + (b1 ? 1 : 0);
-    if (!(hl & 1) && row < nr) done(row, v);
+    if (!(hl & 1) && row < nr) done(row, v.value());
   }
 }
 
@@ -168,89 +190,6 @@ __global__ void k_trace_gather(const int* fs_elem, const int* fs_loc, int64_t F,
   }
 }
 
-// w_e = S_e x_e from the double-float copy of S, in double-float arithmetic on the FP32 pipe
-// (exact products by FMA residuals, two-sum accumulation; ~2^-46 relative per product). S streams
-// through shared memory by bulk asynchronous copies: a persistent CTA walks its elements
-// (e = blockIdx.x, + gridDim.x, ...) in chunks of CR rows (the last one ragged); thread 0 keeps
-// kMvStages chunks in flight on an mbarrier ring and refills a slot once every warp has passed it;
-// the warps read rows from shared memory (row r: lanes over columns, then a warp sum). No thread
-// issues a global load of S, so the copy engine sets the pace. A wait that gives up (about a
-// second) sets *err, writes NaN for the element and ends the CTA once its own copies have drained
-// (bounded as well).
-constexpr int kMvStages = 4;
-constexpr int kMvCtasPerSm = 3;
-constexpr int kMvChunkBytes = 12800;
-constexpr int kMvWaitPolls = 4 * 1000 * 1000;  // ~1 s at 256 ns per poll
-__global__ void __launch_bounds__(256) k_elem_matvec_df(const df2* __restrict__ Sdf, const double* x,
-                                                        const int* tgidx, int64_t E, int NT, int M, int CR,
-                                                        int nchunk, double* w, int* err, const int* skip) {
-  if (skip && *skip) return;  // a finished Krylov cycle: nothing to do
-  extern __shared__ __align__(128) df2 smf[];
-  __shared__ uint64_t full[kMvStages];
-  __shared__ int s_fail;
-  const size_t chunk_entries = (size_t)CR * NT;
-  df2* xs = smf + kMvStages * chunk_entries;  // [NT]
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  const int64_t my_elems = blockIdx.x < E ? (E - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-  const int64_t Q = my_elems * nchunk;  // chunks of this CTA, in order
-  if (Q == 0) return;
-  auto chunk_rows = [&](int k) { return k == nchunk - 1 ? NT - (nchunk - 1) * CR : CR; };
-  auto issue = [&](int64_t q) {  // thread 0: chunk q into slot q % kMvStages
-    const int64_t e = blockIdx.x + (q / nchunk) * gridDim.x;
-    const int k = (int)(q % nchunk);
-    const uint32_t bytes = (uint32_t)(sizeof(df2) * chunk_rows(k) * NT);
-    uint64_t* bar = full + (q % kMvStages);
-    mbar_arrive_expect_tx(bar, bytes);
-    bulk_g2s(smf + (q % kMvStages) * chunk_entries, Sdf + (e * NT + (int64_t)k * CR) * NT, bytes, bar);
-  };
-  if (tid == 0) {
-    for (int i = 0; i < kMvStages; ++i) mbar_init(full + i, 1);
-    fence_mbar_init();
-  }
-  __syncthreads();
-  int64_t issued = 0;
-  if (tid == 0)
-    for (; issued < Q && issued < kMvStages; ++issued) issue(issued);
-  for (int64_t q = 0; q < Q; ++q) {
-    const int64_t e = blockIdx.x + (q / nchunk) * gridDim.x;
-    const int k = (int)(q % nchunk);
-    if (tid == 0) s_fail = 0;
-    if (k == 0) {  // the element's x, gathered once (the previous element is done with xs)
-      const int nfc = NT / M;
-      for (int t = tid; t < NT; t += blockDim.x) xs[t] = df_from(x[(int64_t)tgidx[e * nfc + t / M] * M + t % M]);
-    }
-    __syncthreads();
-    if (!mbar_wait(full + (q % kMvStages), (uint32_t)((q / kMvStages) & 1), kMvWaitPolls)) s_fail = 1;
-    __syncthreads();
-    if (s_fail) {  // give up: NaN for the element, let the copies in flight land, leave
-      for (int t = tid; t < NT; t += blockDim.x) w[e * NT + t] = __longlong_as_double(0x7ff8000000000000LL);
-      if (tid == 0) {
-        atomicExch(err, 1);
-        for (int64_t p = q; p < issued; ++p)
-          mbar_wait(full + (p % kMvStages), (uint32_t)((p / kMvStages) & 1), kMvWaitPolls);
-      }
-      return;
-    }
-    const int rows = chunk_rows(k);
-    const df2* chunk = smf + (q % kMvStages) * chunk_entries;
-    for (int r = wid; r < rows; r += nw) {
-      dfacc a;
-      for (int c = lane; c < NT; c += 32) a.mac(chunk[r * NT + c], xs[c]);
-      for (int off = 16; off > 0; off >>= 1) {
-        const float oh = __shfl_down_sync(0xffffffffu, a.hi, off), ol = __shfl_down_sync(0xffffffffu, a.lo, off);
-        a.add(df2{oh, ol});
-      }
-      if (lane == 0) w[e * NT + (int64_t)k * CR + r] = a.value();
-    }
-    __syncthreads();  // every warp is done with the slot (and with xs for the last chunk)
-    if (tid == 0 && issued < Q) {
-      fence_proxy_async();
-      issue(issued);
-      ++issued;
-    }
-  }
-}
-
 // EDG (continuous trace): out[t][i] = scale * sum over the local occurrences o of node t of
 // ge[o * M + i], o = e NF NFN + f NFN + c (CSR ptr / occ)
 __global__ void k_node_gather(const int* ptr, const int* occ, int64_t nnode, int M, const double* ge, double scale,
@@ -278,14 +217,117 @@ __global__ void k_elem_matvec(const double* S, const double* x, const int* tgidx
     xs[t] = x[(int64_t)tgidx[e * nfc + fc] * M + i];
   }
   __syncthreads();
-  rows_times_vector(S + e * (int64_t)NT * NT, NT, NT, xs, [&](int r, double v) { w[e * NT + r] = v; });
+  rows_times_vector<RowF64>(S + e * (int64_t)NT * NT, NT, NT, xs, [&](int r, double v) { w[e * NT + r] = v; });
 }
 
 // The double-float copy of S: entry i = hi + lo (hi = S rounded to FP32, lo = the rest rounded),
 // 8 bytes an entry as in FP64, about 48 significant bits.
-__global__ void k_split_df(const double* S, int64_t n, df2* out) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-    out[t] = df_from(S[t]);
+__global__ void __launch_bounds__(256) k_split_df(const double* S, int64_t n, df2* out) {
+  for (int64_t t = blockIdx.x * (int64_t)1024 + threadIdx.x; t < n; t += (int64_t)gridDim.x * 1024) {
+    double v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = t + 256 * i < n ? S[t + 256 * i] : 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (t + 256 * i < n) out[t + 256 * i] = df_from(v[i]);
+  }
+}
+
+// w_e = S_e x_e from the double-float copy of S, in double-float arithmetic on the FP32 pipe (exact products by FMA
+// residuals, two-sum accumulation; about 2^-46 relative per product). Two forms: small elements as above; large ones
+// (kMvRingNT) through rings of bulk copies.
+__global__ void k_elem_matvec_df(const df2* S, const double* x, const int* tgidx, int NT, int M, double* w,
+                                 const int* skip) {
+  if (skip && *skip) return;  // a finished Krylov cycle: nothing to do
+  extern __shared__ __align__(128) df2 smf[];
+  const int64_t e = blockIdx.x;
+  const int nfc = NT / M;
+  for (int t = threadIdx.x; t < NT; t += blockDim.x) smf[t] = df_from(x[(int64_t)tgidx[e * nfc + t / M] * M + t % M]);
+  __syncthreads();
+  rows_times_vector<RowDf>(S + e * (int64_t)NT * NT, NT, NT, smf, [&](int r, double v) { w[e * NT + r] = v; });
+}
+
+// Large elements: a warp walks its own contiguous share of all chunks of eight rows, with its own ring of bulk copies (lane 0
+// issues them) and its own x, so that no warp waits for another. Lanes take columns; the eight sums are folded together
+// while they are added up over the lanes. A wait that gives up (about a second) sets *err, writes NaN for the
+// chunk and ends the warp once its copies have drained (bounded as well).
+// HBM bound; 3D p = 3, 3,072 elements (0.98 GB): 170 us, against 298 us with chunks shared by the
+// warps of a CTA and 353 us by rows_times_vector.
+constexpr int kMvRows = 8, kMvWarps = 8, kMvMaxSlots = 4;
+constexpr int kMvWaitPolls = 4 * 1000 * 1000;  // ~1 s at 256 ns per poll
+__global__ void __launch_bounds__(32 * kMvWarps) k_elem_matvec_ring(const df2* __restrict__ Sdf, const double* x,
+                                                                   const int* tgidx, int64_t E, int NT, int M, int slots,
+                                                                   double* w, int* err, const int* skip) {
+  if (skip && *skip) return;  // a finished Krylov cycle: nothing to do
+  extern __shared__ __align__(128) df2 smf[];
+  __shared__ uint64_t bars[kMvWarps][kMvMaxSlots];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nch = (NT + kMvRows - 1) / kMvRows, nfc = NT / M;
+  const int64_t chunks = E * nch, warps = (int64_t)gridDim.x * kMvWarps, g = (int64_t)blockIdx.x * kMvWarps + wid;
+  const int64_t q0 = chunks * g / warps, q1 = chunks * (g + 1) / warps;
+  df2* ring = smf + (size_t)wid * slots * kMvRows * NT;
+  df2* xs = smf + (size_t)kMvWarps * slots * kMvRows * NT + (size_t)wid * NT;
+  uint64_t* full = bars[wid];
+  auto rows_of = [&](int k) { return k == nch - 1 ? NT - (nch - 1) * kMvRows : kMvRows; };
+  auto issue = [&](int64_t q) {  // lane 0: chunk q into its slot
+    const int64_t e = q / nch;
+    const int k = (int)(q % nch), slot = (int)((q - q0) % slots);
+    const uint32_t bytes = (uint32_t)(sizeof(df2) * rows_of(k) * NT);
+    mbar_arrive_expect_tx(full + slot, bytes);
+    bulk_g2s(ring + (size_t)slot * kMvRows * NT, Sdf + (e * NT + (int64_t)k * kMvRows) * NT, bytes, full + slot);
+  };
+  if (lane == 0) {
+    for (int i = 0; i < slots; ++i) mbar_init(full + i, 1);
+    fence_mbar_init();
+    for (int64_t q = q0; q < q1 && q < q0 + slots; ++q) issue(q);
+  }
+  __syncwarp();
+  int64_t cur = -1;
+  for (int64_t q = q0; q < q1; ++q) {
+    const int64_t e = q / nch;
+    const int k = (int)(q % nch), slot = (int)((q - q0) % slots), rows = rows_of(k);
+    if (e != cur) {
+      for (int t = lane; t < NT; t += 32) xs[t] = df_from(x[(int64_t)tgidx[e * nfc + t / M] * M + t % M]);
+      cur = e;
+      __syncwarp();
+    }
+    const bool ok = mbar_wait(full + slot, (uint32_t)(((q - q0) / slots) & 1), kMvWaitPolls);
+    if (!__all_sync(0xffffffffu, ok)) {
+      if (lane < rows) w[e * NT + k * kMvRows + lane] = __longlong_as_double(0x7ff8000000000000LL);
+      if (lane == 0) {
+        atomicExch(err, 1);
+        for (int64_t p = q; p < q1 && p < q + slots; ++p)
+          mbar_wait(full + (p - q0) % slots, (uint32_t)(((p - q0) / slots) & 1), kMvWaitPolls);
+      }
+      return;
+    }
+    const df2* chunk = ring + (size_t)slot * kMvRows * NT;
+    RowDf s[kMvRows];
+#pragma unroll 2
+    for (int c = lane; c < NT; c += 32) {
+      const df2 xc = xs[c];
+#pragma unroll
+      for (int i = 0; i < kMvRows; ++i) s[i].mac(chunk[i * NT + c], xc);  // rows past a ragged chunk are dropped below
+    }
+#pragma unroll
+    for (int m = 4; m > 0; m >>= 1) {  // lane l ends with the sum of row l / 4
+      const bool up = lane & (4 * m);
+#pragma unroll
+      for (int i = 0; i < kMvRows / 2; ++i)
+        if (i < m) {
+          const RowDf give = up ? s[i] : s[i + m];
+          s[i] = up ? s[i + m] : s[i];
+          s[i].fold(give, 4 * m);
+        }
+    }
+    s[0].fold(RowDf(s[0]), 2);
+    s[0].fold(RowDf(s[0]), 1);
+    if (!(lane & 3) && lane / 4 < rows) w[e * NT + k * kMvRows + lane / 4] = s[0].value();
+    __syncwarp();  // all lanes are done with the slot
+    if (lane == 0 && q + slots < q1) {
+      fence_proxy_async();
+      issue(q + slots);
+    }
+  }
 }
 
 // dV_e = -y_e - X_e P_e dVhat
@@ -301,7 +343,7 @@ __global__ void k_recover(const double* recov, const double* dvh, const int* tgi
   __syncthreads();
   const double* X = recov + e * (int64_t)(NV * NT + NV);
   const double* y = X + (int64_t)NV * NT;
-  rows_times_vector(X, NV, NT, xs, [&](int r, double v) { dV[e * NV + r] = -y[r] - v; });
+  rows_times_vector<RowF64>(X, NV, NT, xs, [&](int r, double v) { dV[e * NV + r] = -y[r] - v; });
 }
 
 __global__ void k_sumsq_elem_rows(const double* R, int64_t E, int stride, int n, double* out) {
@@ -821,21 +863,23 @@ int launch_trace_matvec(hdg_ctx* ctx, const double* S, const double* x, double* 
   return launch_gather(ctx, work, y, s, skip);
 }
 
-// y = K x from the double-float copy of S (see k_elem_matvec_df)
-// shared memory of k_elem_matvec_df; its attribute, the SM count and the error flag are set up
-// on first use (before any stream capture: none of these steps may be captured)
-static size_t matvec_df_smem(const hdg_ctx* ctx, int* CR, int* nchunk) {
-  const int NT = ctx->NT;
-  *CR = std::max(1, std::min(NT, kMvChunkBytes / (int)(sizeof(df2) * NT)));
-  *nchunk = (NT + *CR - 1) / *CR;
-  return sizeof(df2) * ((size_t)kMvStages * *CR * NT + NT);
+// y = K x from the double-float copy of S. From kMvRingNT rows on by k_elem_matvec_ring: 30 iterations at 120 rows (3D p = 2, 10,368
+// elements) take 21.5 ms against 24.4, at 200 rows 13.8 against 19.3, but at 60 rows (2D p = 4, 8,192 elements) 8.5 against 7.7.
+// The ring's slots per warp, as many of up to four as fit into an SM's shared memory (0: elements that take the other form).
+constexpr int kMvRingNT = 96;
+static int matvec_ring_slots(const hdg_ctx* ctx, size_t* smem) {
+  const size_t slot = sizeof(df2) * kMvRows * ctx->NT, xs = sizeof(df2) * ctx->NT, room = (size_t)222 * 1024 / kMvWarps;
+  const int n = room < xs ? 0 : (int)std::min<size_t>(kMvMaxSlots, (room - xs) / slot);
+  *smem = kMvWarps * (n * slot + xs);
+  return ctx->NT >= kMvRingNT && n >= 2 && ctx->NT % 2 == 0 ? n : 0;  // copies start on 16 bytes
 }
 
+// the ring's attribute, the SM count and the error flag are set up on first use (before any stream capture: none of
+// these steps may be captured)
 static int prepare_matvec_df(hdg_ctx* ctx) {
-  int CR, nchunk;
-  const size_t smem = matvec_df_smem(ctx, &CR, &nchunk);
-  if (!ctx->attr_matvec) {  // per context, hence per device
-    HDG_CK(cudaFuncSetAttribute(k_elem_matvec_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  size_t smem;
+  if (!ctx->attr_matvec && matvec_ring_slots(ctx, &smem)) {  // per context, hence per device
+    HDG_CK(cudaFuncSetAttribute(k_elem_matvec_ring, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (!ctx->num_sms) HDG_CK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
     if (!ctx->d_mv_err) {
       HDG_CK(cudaMalloc(&ctx->d_mv_err, sizeof(int)));
@@ -849,12 +893,13 @@ static int prepare_matvec_df(hdg_ctx* ctx) {
 static int launch_trace_matvec_df(hdg_ctx* ctx, const df2* Sdf, const double* x, double* y, double* work,
                                   cudaStream_t s, const int* skip = nullptr) {
   if (int rc = prepare_matvec_df(ctx)) return rc;
-  const int NT = ctx->NT;
-  int CR, nchunk;
-  const size_t smem = matvec_df_smem(ctx, &CR, &nchunk);
-  const int64_t grid = std::min<int64_t>(ctx->E, (int64_t)kMvCtasPerSm * ctx->num_sms);
-  k_elem_matvec_df<<<(unsigned)grid, 256, smem, s>>>(Sdf, x, ctx->d_tgidx, ctx->E, NT, ctx->M, CR, nchunk, work,
-                                                      ctx->d_mv_err, skip);
+  size_t smem;
+  if (const int slots = matvec_ring_slots(ctx, &smem))
+    k_elem_matvec_ring<<<(unsigned)ctx->num_sms, 32 * kMvWarps, smem, s>>>(Sdf, x, ctx->d_tgidx, ctx->E, ctx->NT, ctx->M,
+                                                                          slots, work, ctx->d_mv_err, skip);
+  else
+    k_elem_matvec_df<<<(unsigned)ctx->E, row_threads(ctx->NT), sizeof(df2) * ctx->NT, s>>>(Sdf, x, ctx->d_tgidx, ctx->NT,
+                                                                                         ctx->M, work, skip);
   return launch_gather(ctx, work, y, s, skip);
 }
 
@@ -1040,7 +1085,7 @@ static int gmres_solve(hdg_ctx* ctx, const double* S, const double* g, double* x
   const df2* Sdf = nullptr;
   if (ctx->d_Sdf && !ctx->pm) {
     const int64_t ns = (int64_t)ctx->E * ctx->NT * ctx->NT;
-    k_split_df<<<nblocks(ns), kThreads, 0, s>>>(S, ns, static_cast<df2*>(ctx->d_Sdf));
+    k_split_df<<<nblocks(ns, 1024), 256, 0, s>>>(S, ns, static_cast<df2*>(ctx->d_Sdf));
     Sdf = static_cast<const df2*>(ctx->d_Sdf);
   }
   auto arnoldi_matvec = [&](const double* xin, double* yout, cudaStream_t st, const int* skip) {
