@@ -302,8 +302,8 @@ CondVariant make_cond_variant() {
 // 16-column blocks, two CTAs per SM
 template <class C>
 CondVariant make_cond_variant2() {
-  return CondVariant{256, CondTC2<C, 256, kSlices>::bytes, &k_condense_tc2<C, 256, kSlices>, 2,
-                     &k_condense_prep<C, kSlices, false>};
+  using Q = CondTC2<C, 256, kSlices>;
+  return CondVariant{256, Q::bytes, &k_condense_tc2<C, 256, kSlices>, Q::CTAS, &k_condense_prep<C, kSlices, false>};
 }
 
 // tcgen05 products with TMEM accumulators, 32-column blocks, one CTA per SM

@@ -247,7 +247,8 @@ HDG_DEVI bool gj_inverse_reg(float* G, int* si, float* prow) {
 // global memory [NTL][KT][OZS][32]) with the block's X^T (left operand, nmt tiles of 16
 // block columns, sliced in shared memory [KT][NMB][OZS][32]). Each warp owns one tile of 8
 // rows across all the block's columns, so every right-operand fragment is read from L2 once
-// per block; the next k tile's fragments load during this tile's products.
+// per block. The fragments of two k tiles are in flight ahead of a tile's products: one tile's products are shorter
+// than L2's latency (82,944 tetrahedra, p = 3: 232 ms with one tile ahead, 216 with two, 217 with three).
 // epi(row, col, value_without_scales) per element (row of A' or C', block column).
 // The right operand is stored with OZG >= OZS slices per tile; the first OZS are used. With
 // PF each warp asks L2 for its next task's fragments (one contiguous run) while it works.
@@ -270,24 +271,24 @@ HDG_DEVI void cond_oz_product(const uint2* __restrict__ Rsl, int NTL, const uint
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[m][d][q] = 0.f;
     const uint2* Bt = Rsl + (size_t)task * KT * OZG * 32 + lane;
-    uint2 b[OZS], bn[OZS];
+    uint2 b[3][OZS];
 #pragma unroll
-    for (int s = 0; s < OZS; ++s) b[s] = Bt[s * 32];
-#pragma unroll 1
+    for (int kt = 0; kt < (KT < 2 ? KT : 2); ++kt)
+#pragma unroll
+      for (int s = 0; s < OZS; ++s) b[kt][s] = Bt[(kt * OZG + s) * 32];
+#pragma unroll
     for (int kt = 0; kt < KT; ++kt) {
-      if (kt + 1 < KT)  // next tile's fragments in flight during this tile's products
+      if (kt + 2 < KT)
 #pragma unroll
-        for (int s = 0; s < OZS; ++s) bn[s] = Bt[((kt + 1) * OZG + s) * 32];
+        for (int s = 0; s < OZS; ++s) b[(kt + 2) % 3][s] = Bt[((kt + 2) * OZG + s) * 32];
 #pragma unroll
       for (int m = 0; m < NMB; ++m)
         if (m < nmt) {
           uint4 a[OZS];
 #pragma unroll
           for (int s = 0; s < OZS; ++s) a[s] = Xs[((kt * NMB + m) * OZS + s) * 32 + lane];
-          oz_mma_tile<OZS>(acc[m], a, b);
+          oz_mma_tile<OZS>(acc[m], a, b[kt % 3]);
         }
-#pragma unroll
-      for (int s = 0; s < OZS; ++s) b[s] = bn[s];
     }
 #pragma unroll
     for (int m = 0; m < NMB; ++m) {
@@ -637,14 +638,17 @@ __global__ void __launch_bounds__(NTHREADS) k_condense_tc(AssembleArgs a) {
 // of two below its row's (column's) largest, not below itself as FP32 does: with three the
 // small entries of A' lose about two digits against FP32 and X misses 1e-10; four give
 // 2^-33 of the largest, as accurate as the FP32 product. About 108 KB of shared memory, so
-// that two CTAs share an SM and one hides the other's latency. Launched with two CTAs per
-// element (grid 2 ne).
+// that two CTAs share an SM and one hides the other's latency. Launched with CTAS CTAs per
+// element. 82,944 tetrahedra, p = 3: 208 ms, most of it waiting for slices from L2.
 // ------------------------------------------------------------------------------------
 template <class C, int NTHREADS, int OZS>
 struct CondTC2 {
   static constexpr int NV = C::NV, NT = C::NT;
   static constexpr int KT = (NV + 15) / 16, MTA = KT, MTC = (NT + 15) / 16;
   static constexpr int CB = 16, NMB = 1;
+  // CTAs per element: one per two blocks of right-hand sides (3D p = 3: 7 of them; with 2 of them 216 ms instead of
+  // 208 on 82,944 elements, and 2.08 ms instead of 1.95 on 750, whose last wave is then longer)
+  static constexpr int CTAS = ((NT + CB) / CB + 1) / 2;
   static constexpr int RT = 2, CT = 4;
   static constexpr int LDA = (NV + 3) / 4 * 4;
   static constexpr int NTA = (NV + 7) / 8, NTC = (NT + 7) / 8;
@@ -682,10 +686,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_condense_tc2(AssembleArgs a) {
   int* eX = eC + MTC * 16;                                                          // [CB]
   __shared__ int s_bad;
   __shared__ float s_corr[2], s_xmax;
-  // two CTAs per element, on the even and the odd blocks of right-hand sides: the slices of
-  // A' and C' that every block re-reads are then live for half as many elements at a time
-  const int64_t le = blockIdx.x >> 1;
-  const int half = (int)(blockIdx.x & 1);
+  // several CTAs per element, each on every CTAS-th block of right-hand sides: the slices of
+  // A' and C' that every block re-reads are then live for few elements at a time
+  const int64_t le = blockIdx.x / Q::CTAS;
+  const int part = (int)(blockIdx.x % Q::CTAS);
   const int64_t e = a.e0 + le;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint2* slA = reinterpret_cast<const uint2*>(a.oz) + le * P::slice_u2;
@@ -744,8 +748,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_condense_tc2(AssembleArgs a) {
       if (t < NV * CB) W[t] = (bv[x].hi + bv[x].lo) * sc[t / CB];
     }
   };
-  if (half * CB < NT + 1) w_init(half * CB);
-  for (int c0 = half * CB; c0 < NT + 1; c0 += 2 * CB) {
+  if (part * CB < NT + 1) w_init(part * CB);
+  for (int c0 = part * CB; c0 < NT + 1; c0 += Q::CTAS * CB) {
     const int nc = (NT + 1 - c0) < CB ? (NT + 1 - c0) : CB;
     // the block's D' columns, read by the Schur epilogue, copied in the background meanwhile
     for (int t = tid; t < NT * CB; t += NTHREADS) {
@@ -887,7 +891,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_condense_tc2(AssembleArgs a) {
     });
     // W is free since the last correction: warps done with their Schur tasks fill it for
     // this CTA's next block while the others finish
-    if (c0 + 2 * CB < NT + 1) w_init(c0 + 2 * CB);
+    if (c0 + Q::CTAS * CB < NT + 1) w_init(c0 + Q::CTAS * CB);
     __syncthreads();
   }
   if (tid == 0 && s_bad) atomicOr(a.status + e, s_bad);
