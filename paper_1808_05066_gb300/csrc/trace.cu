@@ -573,18 +573,23 @@ __global__ void k_multiaxpy_add_dev(int64_t n, const double* basis, int64_t ld, 
 }
 
 // ---------------------------------------------------------------- face-block Jacobi
-// K_FF (canonical order) = sum_sides S_e[loc rows, loc cols]; LU with partial pivoting, then
-// the inverse column by column (thread t: K_FF x = e_t), stored transposed, fac[F][j][i] =
-// K_FF^{-1}[i][j], so that applying it reads whole rows of fac (B <= kMaxFaceBlock).
+// K_FF (canonical order) = sum_sides S_e[loc rows, loc cols]; its inverse by Gauss-Jordan elimination in place with
+// partial pivoting, stored transposed, fac[F][j][i] = K_FF^{-1}[i][j], so that applying it reads whole rows of fac
+// (B <= kMaxFaceBlock). Two threads per column, odd and even rows; bound by the FP64 pipe (B^3 FMA per face) with enough
+// small blocks on an SM to hide the three barriers per step. The reciprocal of the pivot is formed by one warp: by all
+// threads it takes as long on that pipe as the elimination. 6,144 faces of 50 unknowns: 2.0 ms (LU and the inverse
+// column by column, one thread each: 3.7 ms).
 constexpr int kMaxFaceBlock = 64;
-__global__ void k_face_block_factor(const double* S, const int* fs_elem, const int* fs_loc, int NFN, int M, int NT,
-                                    double* fac) {
-  extern __shared__ double A[];  // [B][B], then X [B][B] (column t of the inverse in X[.][t])
-  __shared__ int s_p;
-  __shared__ int s_piv[kMaxFaceBlock];
-  const int B = NFN * M;
+__global__ void __launch_bounds__(2 * kMaxFaceBlock) k_face_block_inverse(const double* S, const int* fs_elem,
+                                                                          const int* fs_loc, int NFN, int M, int NT,
+                                                                          double* fac) {
+  extern __shared__ double A[];  // [B][B]
+  __shared__ double fcol[kMaxFaceBlock];
+  __shared__ double s_inv;
+  __shared__ int s_piv[kMaxFaceBlock], s_col[kMaxFaceBlock];
+  const int B = NFN * M, tid = threadIdx.x, j = tid >> 1, h = tid & 1;
   const int64_t Fi = blockIdx.x;
-  for (int t = threadIdx.x; t < B * B; t += blockDim.x) {
+  for (int t = tid; t < B * B; t += blockDim.x) {
     int r = t / B, c = t % B;
     int cr = r / M, ir = r % M, cc = c / M, ic = c % M;
     double s = 0.0;
@@ -599,76 +604,53 @@ __global__ void k_face_block_factor(const double* S, const int* fs_elem, const i
   }
   __syncthreads();
   for (int k = 0; k < B; ++k) {
-    if (threadIdx.x < 32) {
-      double best = -1.0;
-      int bi = k;
-      for (int r = k + threadIdx.x; r < B; r += 32) {
-        double v = fabs(A[r * B + k]);
-        if (v > best) {
-          best = v;
-          bi = r;
+    if (tid < 32) {  // the largest |entry| of column k from row k on, the lowest row on ties, and its reciprocal
+      unsigned long long key = 0;
+      int p = INT_MAX;
+      for (int r = k + tid; r < B; r += 32) {
+        const unsigned long long v = lu_key(A[r * B + k]);
+        if (v > key) {
+          key = v;
+          p = r;
         }
       }
-      for (int off = 16; off > 0; off >>= 1) {
-        double ob = __shfl_down_sync(0xffffffffu, best, off);
-        int oi = __shfl_down_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) {
-          best = ob;
-          bi = oi;
-        }
-      }
-      if (threadIdx.x == 0) {
-        s_p = bi;
-        s_piv[k] = bi;
+      lu_warp_max(key, p);
+      if (key == 0) p = k;  // no comparable entry (NaN): no interchange
+      const double d = A[p * B + k], r = d != 0.0 ? 1.0 / d : 0.0;
+      if (tid == 0) {
+        s_piv[k] = p;
+        s_inv = r;
       }
     }
     __syncthreads();
-    int p = s_p;
-    if (p != k)
-      for (int j = threadIdx.x; j < B; j += blockDim.x) {
-        double t = A[k * B + j];
-        A[k * B + j] = A[p * B + j];
-        A[p * B + j] = t;
+    const int p = s_piv[k];
+    const double inv = s_inv;
+    double a = 0.0, old = 0.0;  // row k after the interchange, scaled; and before it: row p after it
+    if (j < B) {
+      a = j == k ? inv : A[p * B + j] * inv;
+      old = A[k * B + j];
+    }
+    if (tid < B) fcol[tid] = tid == p ? A[k * B + k] : A[tid * B + k];
+    __syncthreads();
+    if (j < B) {
+      for (int r = h; r < B; r += 2) {
+        if (r == k) continue;
+        A[r * B + j] = (j == k ? 0.0 : r == p ? old : A[r * B + j]) - fcol[r] * a;
       }
-    __syncthreads();
-    double d = A[k * B + k];
-    double inv = d != 0.0 ? 1.0 / d : 0.0;
-    for (int r = k + 1 + threadIdx.x; r < B; r += blockDim.x) A[r * B + k] *= inv;
-    __syncthreads();
-    int rem = B - k - 1;
-    for (int t = threadIdx.x; t < rem * rem; t += blockDim.x) {
-      int r = k + 1 + t / rem, c = k + 1 + t % rem;
-      A[r * B + c] -= A[r * B + k] * A[k * B + c];
+      if (h == (k & 1)) A[k * B + j] = a;
     }
     __syncthreads();
   }
-  double* X = A + B * B;
-  for (int t = threadIdx.x; t < B; t += blockDim.x) {  // column t of the inverse
-    for (int i = 0; i < B; ++i) X[i * B + t] = i == t ? 1.0 : 0.0;
-    for (int k = 0; k < B; ++k) {  // the row swaps of the factorisation, in order
-      const int p = s_piv[k];
-      if (p != k) {
-        const double tmp = X[k * B + t];
-        X[k * B + t] = X[p * B + t];
-        X[p * B + t] = tmp;
-      }
-    }
-    for (int k = 0; k < B; ++k) {  // unit lower triangle
-      const double xk = X[k * B + t];
-      for (int r = k + 1; r < B; ++r) X[r * B + t] -= A[r * B + k] * xk;
-    }
-    for (int k = B - 1; k >= 0; --k) {  // upper triangle
-      const double d = A[k * B + k];
-      const double xk = d != 0.0 ? X[k * B + t] / d : 0.0;
-      X[k * B + t] = xk;
-      for (int r = 0; r < k; ++r) X[r * B + t] -= A[r * B + k] * xk;
+  if (tid == 0) {  // the row interchanges as column interchanges of the inverse, last one first
+    for (int c = 0; c < B; ++c) s_col[c] = c;
+    for (int k = B - 1; k >= 0; --k) {
+      const int c = s_col[k];
+      s_col[k] = s_col[s_piv[k]];
+      s_col[s_piv[k]] = c;
     }
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < B * B; t += blockDim.x) {
-    const int j = t / B, i = t % B;
-    fac[Fi * (int64_t)B * B + t] = X[i * B + j];
-  }
+  for (int t = tid; t < B * B; t += blockDim.x) fac[Fi * (int64_t)B * B + t] = A[t % B * B + s_col[t / B]];
 }
 
 // z_F = K_FF^{-1} r_F from the stored inverse (fac[F][j][i] = K_FF^{-1}[i][j]), one warp per face:
@@ -863,8 +845,9 @@ int launch_trace_matvec(hdg_ctx* ctx, const double* S, const double* x, double* 
   return launch_gather(ctx, work, y, s, skip);
 }
 
-// y = K x from the double-float copy of S. From kMvRingNT rows on by k_elem_matvec_ring: 30 iterations at 120 rows (3D p = 2, 10,368
-// elements) take 21.5 ms against 24.4, at 200 rows 13.8 against 19.3, but at 60 rows (2D p = 4, 8,192 elements) 8.5 against 7.7.
+// y = K x from the double-float copy of S. From kMvRingNT rows on by k_elem_matvec_ring: 30 iterations at 120 rows
+// (3D p = 2, 10,368 elements) take 21.5 ms against 24.4, at 200 rows (3,072 elements) 13.8 against 19.3, but at 60 rows
+// (2D p = 4, 8,192 elements) 8.5 against 7.7.
 // The ring's slots per warp, as many of up to four as fit into an SM's shared memory (0: elements that take the other form).
 constexpr int kMvRingNT = 96;
 static int matvec_ring_slots(const hdg_ctx* ctx, size_t* smem) {
@@ -1046,7 +1029,7 @@ static int gmres_solve(hdg_ctx* ctx, const double* S, const double* g, double* x
   } else if (ctx->scheme) {
     if (!ctx->d_pcn) HDG_CK(cudaMalloc(&ctx->d_pcn, sizeof(double) * ctx->n_tnodes * ctx->M * ctx->M));
   } else {
-    if (B > kMaxFaceBlock || 2 * sizeof(double) * B * B > 48 * 1024) {  // factor + inverse in shared memory
+    if (B > kMaxFaceBlock || 2 * sizeof(double) * B * B > 48 * 1024) {
       set_error("trace_solve: face block larger than the preconditioner supports");
       return HDG_ERR_UNSUPPORTED;
     }
@@ -1065,8 +1048,8 @@ static int gmres_solve(hdg_ctx* ctx, const double* S, const double* g, double* x
     k_node_block_factor<<<nblocks(ctx->n_tnodes), kThreads, 0, s>>>(S, ctx->d_tr_ptr, ctx->d_tr_occ, ctx->n_tnodes,
                                                                     ctx->M, ctx->NT, ctx->d_pcn);
   else  // HDG: face-block Jacobi
-    k_face_block_factor<<<(unsigned)ctx->F, 64, 2 * sizeof(double) * B * B, s>>>(S, ctx->d_fs_elem, ctx->d_fs_loc,
-                                                                               ctx->NFN, ctx->M, ctx->NT, ctx->d_pc);
+    k_face_block_inverse<<<(unsigned)ctx->F, (2 * B + 31) / 32 * 32, sizeof(double) * B * B, s>>>(
+        S, ctx->d_fs_elem, ctx->d_fs_loc, ctx->NFN, ctx->M, ctx->NT, ctx->d_pc);
   // the double-float copy of S for the Arnoldi products (the restart and final residuals use S
   // itself); without room for it every product is the FP64 one
   const size_t sdf_bytes = sizeof(df2) * (size_t)ctx->E * ctx->NT * ctx->NT;
