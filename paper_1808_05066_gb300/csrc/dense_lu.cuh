@@ -7,7 +7,7 @@
 // tiles stay zero for a while.
 // The FP64 pipe (two FMA per clock and SM) bounds every part: one CTA alone takes 91 us for a panel of 2,304 rows
 // and 2.8 ms for the solves, which is why both are spread over a cluster (25 us, 2.1 ms).
-// 2,304 unknowns (8 x 8 x 2 triangles, p = 2): an implicit Euler step with three factorisations takes 45 ms; with three
+// 2,304 unknowns (8 x 8 x 2 triangles, p = 2): an implicit Euler step with three factorisations takes 42 ms; with three
 // launches per column, a rank-1 update of the whole remainder each and solves one row per barrier, 124 ms.
 #pragma once
 #include <climits>
@@ -230,18 +230,17 @@ __global__ void __launch_bounds__(256) k_lu_inner(double* K, int64_t n, int64_t 
   }
 }
 
-// Columns outside the block [b0, b1), one thread each: the block's interchanges, and behind it the 32 x 32 unit
-// lower triangle. The first warp follows the interchanges on row numbers, so that all of a column's entries are loaded
-// together (interchange by interchange on the entries: 31 us per launch, the latencies of 32 dependent pairs of loads).
-// flag[c / 32]: whether any of these columns' U entries is nonzero. One warp per CTA: the triangle's FMAs share a slow FP64
-// pipe.
-__global__ void __launch_bounds__(32) k_lu_swap(double* K, int64_t n, int64_t b0, int64_t b1, const int* piv,
-                                                     int* flag) {
+// Columns outside the block [b0, b1), 32 per CTA, four lanes each: the block's interchanges, and behind it the 32 x 32
+// unit lower triangle. The first warp follows the interchanges on row numbers, so that all of a column's entries are
+// loaded together. A lane holds every fourth row of its column: a warp's FP64 instruction takes 64 clocks on its own
+// quarter of the SM, so the triangle is spread over all four quarters (15 us per launch; one lane per column 30).
+// flag[c / 32]: whether any of these columns' U entries is nonzero.
+__global__ void __launch_bounds__(128) k_lu_swap(double* K, int64_t n, int64_t b0, int64_t b1, const int* piv, int* flag) {
+  constexpr int NR = kLuBlock / 4;
   __shared__ double L[kLuBlock][kLuBlock + 1];
   __shared__ int src[kLuBlock], orow[kLuBlock], osrc[kLuBlock], s_no;
-  const int w = (int)(b1 - b0), tid = threadIdx.x;
-  const int64_t c = blockIdx.x * (int64_t)32 + tid;
-  {
+  const int w = (int)(b1 - b0), tid = threadIdx.x, lane = tid & 31;
+  if (tid < 32) {
     const int p = tid < w ? piv[b0 + tid] : (int)b0 + tid;
     const int owner = __ffs(__match_any_sync(0xffffffffu, p)) - 1;  // the first interchange with this row
     int in = (int)b0 + tid, out = p;                                // what rows b0 + tid and p hold
@@ -266,38 +265,46 @@ __global__ void __launch_bounds__(32) k_lu_swap(double* K, int64_t n, int64_t b0
       osrc[q] = out;
     }
     if (tid == 0) s_no = __popc(mask);
-  }
-  if ((blockIdx.x + 1) * (int64_t)32 > b1) {
-#pragma unroll
-    for (int t = 0; t < kLuBlock; ++t) L[t][tid] = t < w && tid < w ? K[(b0 + t) * n + b0 + tid] : 0.0;
+  } else if ((blockIdx.x + 1) * (int64_t)32 > b1) {
+    for (int t = tid - 32; t < kLuBlock * kLuBlock; t += 96) {
+      const int r = t / kLuBlock, c = t % kLuBlock;
+      L[r][c] = r < w && c < r ? K[(b0 + r) * n + b0 + c] : 0.0;
+    }
   }
   __syncthreads();
-  bool nz = false;
-  if (c < n && (c < b0 || c >= b1)) {
-    const int no = s_no;
-    double u[kLuBlock], o[kLuBlock];
+  const int col = lane & 7, rg = lane >> 3;  // rows b0 + 4 i + rg
+  const int64_t c = blockIdx.x * (int64_t)32 + (tid >> 5) * 8 + col;
+  const bool live = c < n && (c < b0 || c >= b1);
+  const int no = s_no;
+  double u[NR], o[NR];
 #pragma unroll
-    for (int j = 0; j < kLuBlock; ++j) {
-      u[j] = j < w ? K[(int64_t)src[j] * n + c] : 0.0;
-      o[j] = j < no ? K[(int64_t)osrc[j] * n + c] : 0.0;
-    }
-#pragma unroll
-    for (int j = 0; j < kLuBlock; ++j) {
-      if (j < no) K[(int64_t)orow[j] * n + c] = o[j];
-      nz = nz || u[j] != 0.0;  // true for NaN
-    }
-    nz = nz && c >= b1;
-    if (nz) {  // a zero column stays zero; rows past w: zero factors
-#pragma unroll
-      for (int t = 0; t < kLuBlock; ++t)
-#pragma unroll
-        for (int j = t + 1; j < kLuBlock; ++j) u[j] -= L[j][t] * u[t];
-    }
-#pragma unroll
-    for (int j = 0; j < kLuBlock; ++j)
-      if (j < w) K[(b0 + j) * n + c] = u[j];
+  for (int i = 0; i < NR; ++i) {
+    const int j = 4 * i + rg;
+    u[i] = live && j < w ? K[(int64_t)src[j] * n + c] : 0.0;
+    o[i] = live && j < no ? K[(int64_t)osrc[j] * n + c] : 0.0;
   }
-  const bool any = __any_sync(0xffffffffu, nz);
+  __syncwarp();  // a column's entries are all loaded before any is stored
+  bool nz = false;
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int j = 4 * i + rg;
+    if (live && j < no) K[(int64_t)orow[j] * n + c] = o[i];
+    nz = nz || u[i] != 0.0;  // true for NaN
+  }
+  nz = nz && c >= b1;
+  if (__any_sync(0xffffffffu, nz)) {  // zero columns stay zero
+#pragma unroll
+    for (int t = 0; t < kLuBlock; ++t) {
+      const double ut = __shfl_sync(0xffffffffu, u[t / 4], (t % 4) * 8 + col);
+#pragma unroll
+      for (int i = t / 4; i < NR; ++i)
+        if (c >= b1 && (i > t / 4 || rg > t % 4)) u[i] -= L[4 * i + rg][t] * ut;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NR; ++i)
+    if (live && 4 * i + rg < w) K[(b0 + 4 * i + rg) * n + c] = u[i];
+  const int any = __syncthreads_or(nz);
   if (tid == 0) flag[blockIdx.x] = any;
 }
 
@@ -435,7 +442,7 @@ inline void enqueue_lu(double* K, int64_t n, int* piv, int* bad, int* flag, cuda
         k_lu_inner<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, s>>>(K, n, k0, w, b1);
       }
     }
-    k_lu_swap<<<(unsigned)((n + 31) / 32), 32, 0, s>>>(K, n, b0, b1, piv, flag);
+    k_lu_swap<<<(unsigned)((n + 31) / 32), 128, 0, s>>>(K, n, b0, b1, piv, flag);
     if (b1 < n) {
       const int t0 = (int)(b1 / kLuTile), nt = tiles - t0;
       k_lu_update<<<dim3(nt, nt), 256, 0, s>>>(K, n, b0, b1, t0, flag);
