@@ -63,6 +63,22 @@ HDG_DEVI double f32_to_f64_bits(float x) {
   return __longlong_as_double((long long)bits);
 }
 
+// df_from on the integer pipe (three FP64 instructions a value bound a pass over a large array): the leading 24
+// bits, rounded half up, and the exact rest, rounded to 24 bits. Zero and |x| in [2^-70, 2^70]; other values take
+// the conversion instructions.
+HDG_DEVI df2 df_from_bits(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ffu) - 1023;
+  if ((b << 1) == 0ull) return {0.f, 0.f};
+  if (e < -70 || e > 70) return df_from(x);
+  const unsigned long long m = (b & 0xfffffffffffffull) | (1ull << 52);
+  const unsigned h = (unsigned)((m + (1ull << 28)) >> 29);                      // at most 2^24
+  const int r = (int)((long long)m - (long long)((unsigned long long)h << 29));  // |r| <= 2^28
+  const int sign = (int)(b >> 63) << 31;
+  const float ph = __int_as_float(((e - 23 + 127) << 23) | sign), pl = __int_as_float(((e - 52 + 127) << 23) | sign);
+  return {__uint2float_rn(h) * ph, __int2float_rn(r) * pl};
+}
+
 // hi + lo of a double-float in FP64: one FP64 addition.
 HDG_DEVI double df_to_f64(float hi, float lo) { return f32_to_f64_bits(hi) + f32_to_f64_bits(lo); }
 
