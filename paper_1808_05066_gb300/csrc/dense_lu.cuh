@@ -7,7 +7,7 @@
 // tiles stay zero for a while.
 // The FP64 pipe (two FMA per clock and SM) bounds every part: one CTA alone takes 91 us for a panel of 2,304 rows
 // and 2.8 ms for the solves, which is why both are spread over a cluster (25 us, 2.1 ms).
-// 2,304 unknowns (8 x 8 x 2 triangles, p = 2): an implicit Euler step with three factorisations takes 42 ms; with three
+// 2,304 unknowns (8 x 8 x 2 triangles, p = 2): an implicit Euler step with three factorisations takes 34 ms; with three
 // launches per column, a rank-1 update of the whole remainder each and solves one row per barrier, 124 ms.
 #pragma once
 #include <climits>
@@ -218,7 +218,7 @@ __global__ void __cluster_dims__(kLuCluster, 1, 1) __launch_bounds__(256)
     if (j < w) K[(k0 + j) * n + c] = u[j];
 }
 
-// rows below the panel, columns [k0 + w, b1): -= L U
+// rows below the w columns at k0, columns [k0 + w, b1): -= L U
 __global__ void __launch_bounds__(256) k_lu_inner(double* K, int64_t n, int64_t k0, int w, int64_t b1) {
   const int nc = (int)(b1 - k0 - w);
   const int64_t tot = (n - k0 - w) * nc;
@@ -230,12 +230,21 @@ __global__ void __launch_bounds__(256) k_lu_inner(double* K, int64_t n, int64_t 
   }
 }
 
+inline unsigned lu_inner_grid(int64_t rows, int64_t cols) {
+  const int64_t blocks = (rows * cols + 255) / 256;
+  return (unsigned)(blocks < 152 * 8 ? blocks : 152 * 8);
+}
+
 // Columns outside the block [b0, b1), 32 per CTA, four lanes each: the block's interchanges, and behind it the 32 x 32
 // unit lower triangle. The first warp follows the interchanges on row numbers, so that all of a column's entries are
 // loaded together. A lane holds every fourth row of its column: a warp's FP64 instruction takes 64 clocks on its own
 // quarter of the SM, so the triangle is spread over all four quarters (15 us per launch; one lane per column 30).
 // flag[c / 32]: whether any of these columns' U entries is nonzero.
-__global__ void __launch_bounds__(128) k_lu_swap(double* K, int64_t n, int64_t b0, int64_t b1, const int* piv, int* flag) {
+// Columns 32 (first + blockIdx.x) .., not those of group `skip`.
+__global__ void __launch_bounds__(128) k_lu_swap(double* K, int64_t n, int64_t b0, int64_t b1, const int* piv, int* flag,
+                                                 int first, int skip) {
+  const int group = first + (int)blockIdx.x;
+  if (group == skip) return;
   constexpr int NR = kLuBlock / 4;
   __shared__ double L[kLuBlock][kLuBlock + 1];
   __shared__ int src[kLuBlock], orow[kLuBlock], osrc[kLuBlock], s_no;
@@ -265,7 +274,7 @@ __global__ void __launch_bounds__(128) k_lu_swap(double* K, int64_t n, int64_t b
       osrc[q] = out;
     }
     if (tid == 0) s_no = __popc(mask);
-  } else if ((blockIdx.x + 1) * (int64_t)32 > b1) {
+  } else if ((group + 1) * (int64_t)32 > b1) {
     for (int t = tid - 32; t < kLuBlock * kLuBlock; t += 96) {
       const int r = t / kLuBlock, c = t % kLuBlock;
       L[r][c] = r < w && c < r ? K[(b0 + r) * n + b0 + c] : 0.0;
@@ -273,7 +282,7 @@ __global__ void __launch_bounds__(128) k_lu_swap(double* K, int64_t n, int64_t b
   }
   __syncthreads();
   const int col = lane & 7, rg = lane >> 3;  // rows b0 + 4 i + rg
-  const int64_t c = blockIdx.x * (int64_t)32 + (tid >> 5) * 8 + col;
+  const int64_t c = group * (int64_t)32 + (tid >> 5) * 8 + col;
   const bool live = c < n && (c < b0 || c >= b1);
   const int no = s_no;
   double u[NR], o[NR];
@@ -305,14 +314,15 @@ __global__ void __launch_bounds__(128) k_lu_swap(double* K, int64_t n, int64_t b
   for (int i = 0; i < NR; ++i)
     if (live && 4 * i + rg < w) K[(b0 + 4 * i + rg) * n + c] = u[i];
   const int any = __syncthreads_or(nz);
-  if (tid == 0) flag[blockIdx.x] = any;
+  if (tid == 0) flag[group] = any;
 }
 
-// trailing update K[r][c] -= sum_j L[r][b0 + j] U[b0 + j][c], r, c >= b1, one 64 x 64 tile per CTA
-__global__ void __launch_bounds__(256) k_lu_update(double* K, int64_t n, int64_t b0, int64_t b1, int tile0,
+// trailing update K[r][c] -= sum_j L[r][b0 + j] U[b0 + j][c], r >= b1, c >= cl (a multiple of 32), one 64 x 64 tile per CTA
+__global__ void __launch_bounds__(256) k_lu_update(double* K, int64_t n, int64_t b0, int64_t b1, int64_t cl,
                                                    const int* flag) {
-  const int ct = tile0 + blockIdx.x, rt = tile0 + blockIdx.y;
-  if (!flag[2 * ct] && (2 * ct + 1 >= (n + 31) / 32 || !flag[2 * ct + 1])) return;
+  const int ct = (int)(cl / kLuTile) + blockIdx.x, rt = (int)(b1 / kLuTile) + blockIdx.y;
+  const bool left = 2 * ct * 32 >= cl && flag[2 * ct], right = 2 * ct + 1 < (n + 31) / 32 && flag[2 * ct + 1];
+  if (!left && !right) return;
   __shared__ double A[kLuBlock][kLuTile + 2], B[kLuBlock][kLuTile + 2];  // [j][row], [j][column]
   const int w = (int)(b1 - b0), tid = threadIdx.x;
   const int64_t r0 = (int64_t)rt * kLuTile, c0 = (int64_t)ct * kLuTile;
@@ -327,7 +337,7 @@ __global__ void __launch_bounds__(256) k_lu_update(double* K, int64_t n, int64_t
   if (!__syncthreads_or(nz)) return;
   for (int t = tid; t < kLuTile * kLuBlock; t += 256) {
     const int c = t % kLuTile, j = t / kLuTile;
-    B[j][c] = j < w && c0 + c >= b1 && c0 + c < n ? K[(b0 + j) * n + c0 + c] : 0.0;
+    B[j][c] = j < w && c0 + c >= cl && c0 + c < n ? K[(b0 + j) * n + c0 + c] : 0.0;
   }
   __syncthreads();
   const int ty = tid / 16, tx = tid % 16;  // rows 4 ty .., columns 2 tx, 2 tx + 1, 32 + 2 tx, 32 + 2 tx + 1
@@ -349,7 +359,7 @@ __global__ void __launch_bounds__(256) k_lu_update(double* K, int64_t n, int64_t
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int64_t r = r0 + 4 * ty + i, c = c0 + (q >> 1) * 32 + 2 * tx + (q & 1);
-      if (r >= b1 && c >= b1 && r < n && c < n) K[r * n + c] -= acc[i][q];
+      if (r >= b1 && c >= cl && r < n && c < n) K[r * n + c] -= acc[i][q];
     }
 }
 
@@ -429,25 +439,36 @@ __global__ void __cluster_dims__(kLuCluster, 1, 1) __launch_bounds__(256)
     for (int64_t t = tid; t < n; t += 256) x[t] = xs[t];
 }
 
-// The factorisation's launches on `s`; flag: [n / 32 + 1] ints of scratch.
-inline void enqueue_lu(double* K, int64_t n, int* piv, int* bad, int* flag, cudaStream_t s) {
-  const int tiles = (int)((n + kLuTile - 1) / kLuTile);
+// The factorisation's launches, captured from stream `s` with a branch on `side`; flag: [n / 32 + 1] ints of scratch. The
+// next block's columns are brought up to date first, on `s`, so that its panels, which keep eight SMs busy, run beside
+// the interchanges and the update of all others on `side` (the step below: 42 ms with all in a row). Every kernel touches
+// its own columns only; the block's own L is read by both branches and permuted by the next interchanges on `side`,
+// behind the next panels.
+inline cudaError_t enqueue_lu(double* K, int64_t n, int* piv, int* bad, int* flag, cudaStream_t s, cudaStream_t side,
+                              cudaEvent_t panel, cudaEvent_t rest) {
+  auto fine = [e = cudaSuccess](cudaError_t r) mutable { return e = e == cudaSuccess ? r : e; };
+  const int groups = (int)((n + 31) / 32), tiles = (int)((n + kLuTile - 1) / kLuTile);
   for (int64_t b0 = 0; b0 < n; b0 += kLuBlock) {
-    const int64_t b1 = b0 + kLuBlock < n ? b0 + kLuBlock : n;
+    const int64_t b1 = b0 + kLuBlock < n ? b0 + kLuBlock : n, b2 = b1 + kLuBlock < n ? b1 + kLuBlock : n;
     for (int64_t k0 = b0; k0 < b1; k0 += kLuNB) {
       const int w = (int)(b1 - k0 < kLuNB ? b1 - k0 : kLuNB);
       k_lu_panel<<<kLuCluster, 256, lu_panel_smem((int)(n - k0)), s>>>(K, n, k0, w, b0, b1, piv, bad);
-      if (k0 + w < b1) {
-        const int64_t tot = (n - k0 - w) * (b1 - k0 - w), blocks = (tot + 255) / 256;
-        k_lu_inner<<<(unsigned)(blocks < 152 * 8 ? blocks : 152 * 8), 256, 0, s>>>(K, n, k0, w, b1);
-      }
+      if (k0 + w < b1) k_lu_inner<<<lu_inner_grid(n - k0 - w, b1 - k0 - w), 256, 0, s>>>(K, n, k0, w, b1);
     }
-    k_lu_swap<<<(unsigned)((n + 31) / 32), 128, 0, s>>>(K, n, b0, b1, piv, flag);
+    const int next = b1 < n ? (int)(b1 / 32) : -1;
+    fine(cudaEventRecord(panel, s));
+    fine(cudaStreamWaitEvent(side, panel, 0));
     if (b1 < n) {
-      const int t0 = (int)(b1 / kLuTile), nt = tiles - t0;
-      k_lu_update<<<dim3(nt, nt), 256, 0, s>>>(K, n, b0, b1, t0, flag);
+      if (b0 > 0) fine(cudaStreamWaitEvent(s, rest, 0));  // the next columns' share of the last update
+      k_lu_swap<<<1, 128, 0, s>>>(K, n, b0, b1, piv, flag, next, -1);
+      k_lu_inner<<<lu_inner_grid(n - b1, b2 - b1), 256, 0, s>>>(K, n, b0, (int)(b1 - b0), b2);
     }
+    k_lu_swap<<<groups, 128, 0, side>>>(K, n, b0, b1, piv, flag, 0, next);
+    if (b2 < n)
+      k_lu_update<<<dim3(tiles - (int)(b2 / kLuTile), tiles - (int)(b1 / kLuTile)), 256, 0, side>>>(K, n, b0, b1, b2, flag);
+    fine(cudaEventRecord(rest, side));
   }
+  return fine(cudaStreamWaitEvent(s, rest, 0));
 }
 
 }  // namespace hdg

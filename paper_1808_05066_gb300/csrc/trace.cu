@@ -975,13 +975,26 @@ static int dense_solve(hdg_ctx* ctx, const double* S, const double* g, double* d
   if (!ctx->lu_graph_exec) {
     HDG_CK(cudaFuncSetAttribute(k_lu_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lu_panel_smem(kLuMaxN)));
     HDG_CK(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kLuMaxN * (int)sizeof(double)));
-    cudaStream_t cap = nullptr;
-    HDG_CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
+    cudaStream_t cap = nullptr, side = nullptr;
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    int low = 0, high = 0;
     cudaGraph_t graph = nullptr;
-    HDG_CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-    enqueue_lu(K, n, ctx->d_dpiv, bad, ctx->d_dpiv + n + 1, cap);
-    cudaError_t ce = cudaStreamEndCapture(cap, &graph);
-    cudaStreamDestroy(cap);
+    cudaError_t ce = cudaDeviceGetStreamPriorityRange(&low, &high);
+    if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&cap, cudaStreamNonBlocking, high);
+    if (ce == cudaSuccess) ce = cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, low);
+    for (cudaEvent_t& e : ev)
+      if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+    if (ce == cudaSuccess) ce = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    if (ce == cudaSuccess) {
+      ce = enqueue_lu(K, n, ctx->d_dpiv, bad, ctx->d_dpiv + n + 1, cap, side, ev[0], ev[1]);
+      const cudaError_t end = cudaStreamEndCapture(cap, &graph);
+      if (ce == cudaSuccess) ce = end;
+      if (ce != cudaSuccess && graph) cudaGraphDestroy(graph);
+    }
+    for (cudaEvent_t e : ev)
+      if (e) cudaEventDestroy(e);
+    if (side) cudaStreamDestroy(side);
+    if (cap) cudaStreamDestroy(cap);
     if (ce != cudaSuccess) return cuda_fail(ce, "cudaStreamEndCapture (dense LU)");
     ce = cudaGraphInstantiate(&ctx->lu_graph_exec, graph, 0);
     cudaGraphDestroy(graph);
