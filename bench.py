@@ -254,7 +254,7 @@ def run_reference(args):
 
 def mixed_degree_leg(args, local, barrier, max_over_ranks, ws):
     """Elements/s of the FP64 assemble + condense of the mixed-degree workload (one persistent
-    launch per step over the element classes, tile shapes tuned per class on the first call),
+    launch per step over the element classes),
     with the class census and, on request, one BDF2 Newton step."""
     import torch
     from paper_1808_05066_gb300 import hdg
@@ -264,7 +264,7 @@ def mixed_degree_leg(args, local, barrier, max_over_ranks, ws):
         W = DeviceWorkload(name, device=local, n_override=args.n)
         E = W.info["n_elem"]
         dev = W.dev
-        for _ in range(2):  # the first call tunes the tile shapes
+        for _ in range(2):
             W.status.zero_()
             W.assemble(hdg.HDG_PREC_FP64)
         torch.cuda.synchronize(dev)

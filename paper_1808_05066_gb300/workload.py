@@ -168,11 +168,12 @@ def slice_flops_per_element(info: dict, viscous: bool, kernel: str) -> float:
     2 x rows x columns x contraction length of every nonzero operator block, times the
     S(S+1)/2 slice products. Tile padding and products a kernel shape adds are not counted, so
     this never exceeds what a kernel executes:
-      mixed_assemble: rows (i, l, node) = m^2 NP, contraction NG per operator; the value
+      mixed_assemble: volume: rows (i, l, node) = m^2 NP, contraction NG per operator; the value
                       operator meets the NP interior columns, each of the NR - 1 gradient
-                      operators all NZ;
-      mixed_face:     per face rows m^2 NFN, contraction NGF; value operator NP columns, trace
-                      operator the face's own NFN, each of the NRF - 2 gradient operators all NZ;
+                      operators all NZ; and the faces (one kernel forms both);
+      mixed_face:     the faces' share of it: per face rows m^2 NFN, contraction NGF; value operator
+                      NP columns, trace operator the face's own NFN, each of the NRF - 2
+                      gradient operators all NZ;
       mixed_condense: r0 = B - A' X0 and S = D - C' X: NV + NT rows, NT + 1 right-hand sides,
                       contraction NV."""
     D, M = info["dim"], info["m"]
@@ -182,10 +183,11 @@ def slice_flops_per_element(info: dict, viscous: bool, kernel: str) -> float:
     NR = D + 1 if viscous else 1
     NRF = D + 2 if viscous else 2
     prod = SLICES * (SLICES + 1) // 2
+    face = 2.0 * prod * NF * (M * M * NFN) * NGF * (NP + NFN + (NRF - 2) * NZ)
     if kernel == "mixed_assemble":
-        return 2.0 * prod * (M * M * NP) * NG * (NP + (NR - 1) * NZ)
+        return 2.0 * prod * (M * M * NP) * NG * (NP + (NR - 1) * NZ) + face
     if kernel == "mixed_face":
-        return 2.0 * prod * NF * (M * M * NFN) * NGF * (NP + NFN + (NRF - 2) * NZ)
+        return face
     if kernel == "mixed_condense":
         return 2.0 * prod * (NV + NT) * (NT + 1) * NV
     raise ValueError(kernel)
@@ -193,8 +195,8 @@ def slice_flops_per_element(info: dict, viscous: bool, kernel: str) -> float:
 
 def algorithmic_bytes_per_element(info: dict, kernel: str) -> int:
     """HBM bytes one element needs moved by a mixed-form kernel (8-byte values):
-      mixed_assemble: read the volume point tensors, write A' and B';
-      mixed_face:     read the face point tensors, write C' and D', add into A' and B';
+      mixed_assemble: read the point tensors, write A', B', C' and D';
+      mixed_face:     the share of the face point tensors, C' and D';
       mixed_condense: the method's outputs only: write S, X, y and g (the blocks the assembly
                       parks in HBM for it are this implementation's, not the method's)."""
     D, M = info["dim"], info["m"]
@@ -202,10 +204,11 @@ def algorithmic_bytes_per_element(info: dict, kernel: str) -> int:
     NV, NT = info["nv"], info["nt"]
     pt_vol = M + D * M + M * M + D * M * M + D * M * M * D
     pt_face = M + 2 * M * M + M * M * D
+    face = 8 * (NF * NGF * pt_face + NT * (NV + NT))
     if kernel == "mixed_assemble":
-        return 8 * (NG * pt_vol + NV * (NV + NT))
+        return 8 * (NG * pt_vol + NV * (NV + NT)) + face
     if kernel == "mixed_face":
-        return 8 * (NF * NGF * pt_face + NT * (NV + NT) + 2 * NV * (NV + NT))
+        return face
     if kernel == "mixed_condense":
         return 8 * (NT * NT + NV * NT + NV + NT)
     raise ValueError(kernel)
@@ -213,15 +216,12 @@ def algorithmic_bytes_per_element(info: dict, kernel: str) -> int:
 
 def method_flops_per_element(info: dict, viscous: bool, kernel: str) -> float:
     """The method's own flops per element of a mixed-form kernel, the same count as the FP64
-    form's kernels (flops_per_element): the assembly contractions for mixed_assemble +
-    mixed_face (split by the share of their slice products), the LU, solves and Schur product
-    for mixed_condense."""
+    form's kernels (flops_per_element): the assembly contractions for mixed_assemble (mixed_face: the
+    faces' share by slice products), the LU, solves and Schur product for mixed_condense."""
     if kernel == "mixed_condense":
         return flops_per_element(info, viscous, "condense")
     asm = flops_per_element(info, viscous, "assemble")
-    v = slice_flops_per_element(info, viscous, "mixed_assemble")
-    f = slice_flops_per_element(info, viscous, "mixed_face")
-    return asm * (v if kernel == "mixed_assemble" else f) / (v + f)
+    return asm * slice_flops_per_element(info, viscous, kernel) / slice_flops_per_element(info, viscous, "mixed_assemble")
 
 
 
