@@ -4,21 +4,19 @@
 
 #include "assemble_fp64.cuh"
 #include "ctx.hpp"
+#include "element_small.cuh"
 
 namespace hdg {
 
 namespace {
 
 template <class C>
-size_t scratch_per_element() {
-  return sizeof(double) * ((size_t)C::NG * C::PT_VOL + (size_t)C::NF * C::NGF * C::PT_FACE +
-                           (size_t)C::NV * C::NV + (size_t)C::NT * C::NV);
-}
-
-template <class C>
 int run_fp64(hdg_ctx* ctx, const double* V, const double* Vhat, const double* hist, double mass_coef, double* S,
              double* g, double* recov, double* R, int32_t* status, cudaStream_t s) {
-  const size_t per = scratch_per_element<C>();
+  const bool sm = small::small_elements<C>(ctx->E);
+  size_t vol, face;
+  point_doubles<C>(sm, &vol, &face);
+  const size_t per = sizeof(double) * (vol + face + (size_t)C::NV * C::NV + (size_t)C::NT * C::NV);
   if (ctx->chunk == 0) {
     int64_t ch = std::min<int64_t>(ctx->E, 8192);
     while (ch > 256 && per * ch > ((size_t)3 << 30)) ch /= 2;
@@ -33,8 +31,7 @@ int run_fp64(hdg_ctx* ctx, const double* V, const double* Vhat, const double* hi
     ctx->scr_bytes = need;
   }
   if (!ctx->attr_fp64) {  // per context, hence per device
-    HDG_CK(cudaFuncSetAttribute(k_assemble<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AsmSmem<C>::bytes));
-    HDG_CK(cudaFuncSetAttribute(k_condense<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CondSmem<C>::bytes));
+    if (int rc = fp64_attributes<C>()) return rc;
     ctx->attr_fp64 = true;
   }
   AssembleArgs a{};
@@ -51,8 +48,8 @@ int run_fp64(hdg_ctx* ctx, const double* V, const double* Vhat, const double* hi
   a.status = status;
   const int64_t ch = ctx->chunk;
   a.ptv = ctx->d_scr;
-  a.ptf = a.ptv + ch * C::NG * C::PT_VOL;
-  a.Ap = a.ptf + ch * C::NF * C::NGF * C::PT_FACE;
+  a.ptf = a.ptv + ch * vol;
+  a.Ap = a.ptf + ch * face;
   a.Cp = a.Ap + ch * C::NV * C::NV;
   for (int64_t e0 = 0; e0 < ctx->E; e0 += ch) {
     a.e0 = e0;
@@ -64,16 +61,16 @@ int run_fp64(hdg_ctx* ctx, const double* V, const double* Vhat, const double* hi
     }
     {
       LaunchScope ls(ctx, HDG_KERNEL_POINTWISE, s);
-      launch_pointwise<C>(a, ctx->T, ctx->ph, s);
+      fp64_pointwise<C>(sm, a, ctx->T, ctx->ph, s);
     }
     {
       LaunchScope ls(ctx, HDG_KERNEL_ASSEMBLE, s);
-      k_assemble<C><<<(unsigned)a.ne, AsmSmem<C>::NTH, AsmSmem<C>::bytes, s>>>(a, ctx->T);
+      fp64_assemble<C>(sm, a, ctx->T, s);
     }
     if (int rc_b = boundary_patch(ctx, a, HDG_PREC_FP64, s)) return rc_b;
     {
       LaunchScope ls(ctx, HDG_KERNEL_CONDENSE, s);
-      k_condense<C><<<(unsigned)a.ne, CondSmem<C>::NTH, CondSmem<C>::bytes, s>>>(a);
+      fp64_condense<C>(sm, a, s);
     }
     if (int rc_d = chunk_done(ctx, e0, a.ne, s)) return rc_d;
   }

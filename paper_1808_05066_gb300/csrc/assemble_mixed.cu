@@ -5,6 +5,7 @@
 #include <set>
 #include <vector>
 
+#include "element_small.cuh"
 #include "asm_t5.cuh"
 #include "condense_t5.cuh"
 #include "condense_tc.cuh"
@@ -338,8 +339,13 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
   const T5Plan& pl = *static_cast<T5Plan*>(ctx->t5_plan);
   T5Prog pr[2] = {pl.prog[0], pl.prog[1]};
   using TC = CondTC<C, 256, kSlices>;
-  const size_t per_pt = sizeof(double) * ((size_t)C::NG * C::PT_VOL + (size_t)C::NF * C::NGF * C::PT_FACE +
-                                          (size_t)C::NV * C::NV + (size_t)C::NT * C::NV);
+  // the recomputation of flagged blocks may need more room for its point data
+  const bool sm = small::small_elements<C>(ctx->E);
+  size_t vol, face, rvol, rface;
+  point_doubles<C>(false, &vol, &face);
+  point_doubles<C>(sm, &rvol, &rface);
+  const size_t pts = std::max(vol + face, rvol + rface);
+  const size_t per_pt = sizeof(double) * (pts + (size_t)C::NV * C::NV + (size_t)C::NT * C::NV);
   const size_t slice_bytes = std::max(sizeof(uint4) * TC::slice_uint4, CondT5<C, kSlices>::slice_bytes);
   const size_t per_rows = t5_slice_bytes(pr[0], 1024) / 1024 + t5_slice_bytes(pr[1], 1024) / 1024;
   const size_t per = per_pt + slice_bytes + sizeof(float) * TC::prep_floats + per_rows;
@@ -371,8 +377,7 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     HDG_CK(cudaFuncSetAttribute(k_condense_prep<C, kSlices, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)TC::prep_bytes));
     // the FP64 kernels of the flagged-only recomputation
-    HDG_CK(cudaFuncSetAttribute(k_assemble<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AsmSmem<C>::bytes));
-    HDG_CK(cudaFuncSetAttribute(k_condense<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CondSmem<C>::bytes));
+    if (int rc = fp64_attributes<C>()) return rc;
     ctx->attr_mixed = true;
   }
   AssembleArgs a{};
@@ -391,8 +396,8 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
   a.stall_first_copy = ctx->t5_stall ? 1 : 0;
   const int64_t ch = ctx->chunk;
   a.ptv = ctx->d_scr;
-  a.ptf = a.ptv + ch * C::NG * C::PT_VOL;
-  a.Ap = a.ptf + ch * C::NF * C::NGF * C::PT_FACE;
+  a.ptf = a.ptv + ch * vol;
+  a.Ap = a.ptv + ch * pts;
   a.Cp = a.Ap + ch * C::NV * C::NV;
   {  // 256-byte aligned start of the slice scratch (chunk sizes may be odd)
     const uintptr_t p = reinterpret_cast<uintptr_t>(a.Cp + ch * C::NT * C::NV);
@@ -458,17 +463,23 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     }
     if (ctx->refine_fallback) {
       // blocks whose refinement missed its tolerance (or whose condensation gave up a wait) are
-      // recomputed by the FP64 kernels from the same point tensors; every other CTA returns at once
+      // recomputed by the FP64 kernels, from the same point tensors or those of small elements; every other CTA returns
+      // at once
       AssembleArgs f = a;
       f.only_flag = HDG_STATUS_REFINE | HDG_STATUS_TIMEOUT;
+      if (sm) {
+        f.ptf = f.ptv + ch * rvol;
+        LaunchScope ls(ctx, HDG_KERNEL_POINTWISE, s);
+        fp64_pointwise<C>(sm, f, ctx->T, ctx->ph, s);
+      }
       {
         LaunchScope ls(ctx, HDG_KERNEL_ASSEMBLE, s);
-        k_assemble<C><<<(unsigned)a.ne, AsmSmem<C>::NTH, AsmSmem<C>::bytes, s>>>(f, ctx->T);
+        fp64_assemble<C>(sm, f, ctx->T, s);
       }
       if (int rc_b = boundary_patch(ctx, f, HDG_PREC_FP64, s)) return rc_b;
       {
         LaunchScope ls(ctx, HDG_KERNEL_CONDENSE, s);
-        k_condense<C><<<(unsigned)a.ne, CondSmem<C>::NTH, CondSmem<C>::bytes, s>>>(f);
+        fp64_condense<C>(sm, f, s);
       }
     }
     if (int rc_d = chunk_done(ctx, e0, a.ne, s)) return rc_d;

@@ -24,6 +24,7 @@
 
 #include "assemble_fp64.cuh"
 #include "ctx.hpp"
+#include "element_small.cuh"
 
 namespace {
 
@@ -56,16 +57,17 @@ template <class C>
 int run_noalloc(hdg_ctx* ctx, double* scratch, const double* V, const double* Vhat, const double* hist,
                 double mass_coef, double* S, double* g, double* recov, double* R, int32_t* status, cudaStream_t s) {
   using namespace hdg;
-  const size_t per = (size_t)C::NG * C::PT_VOL + (size_t)C::NF * C::NGF * C::PT_FACE + (size_t)C::NV * C::NV +
-                     (size_t)C::NT * C::NV;  // doubles per element
+  const bool sm = small::small_elements<C>(ctx->E);
+  size_t vol, face;
+  point_doubles<C>(sm, &vol, &face);
+  const size_t per = vol + face + (size_t)C::NV * C::NV + (size_t)C::NT * C::NV;  // doubles per element
   const int64_t ch = std::min<int64_t>(ctx->E, (int64_t)(kNoAllocScratchBytes / sizeof(double) / per));
   if (ch < 1) {
     set_error("hdg_assemble_condense_noalloc: one element needs more scratch than the 64 MiB static array");
     return HDG_ERR_INVALID_ARG;
   }
   if (!ctx->attr_noalloc) {  // this file's instances of the kernels, once per context (one device)
-    HDG_CK(cudaFuncSetAttribute(k_assemble<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AsmSmem<C>::bytes));
-    HDG_CK(cudaFuncSetAttribute(k_condense<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CondSmem<C>::bytes));
+    if (int rc = fp64_attributes<C>()) return rc;
     ctx->attr_noalloc = true;
   }
   AssembleArgs a{};
@@ -81,16 +83,16 @@ int run_noalloc(hdg_ctx* ctx, double* scratch, const double* V, const double* Vh
   a.R = R;
   a.status = status;
   a.ptv = scratch;
-  a.ptf = a.ptv + ch * C::NG * C::PT_VOL;
-  a.Ap = a.ptf + ch * C::NF * C::NGF * C::PT_FACE;
+  a.ptf = a.ptv + ch * vol;
+  a.Ap = a.ptf + ch * face;
   a.Cp = a.Ap + ch * C::NV * C::NV;
   for (int64_t e0 = 0; e0 < ctx->E; e0 += ch) {
     a.e0 = e0;
     a.ne = std::min<int64_t>(ch, ctx->E - e0);
-    launch_pointwise<C>(a, ctx->T, ctx->ph, s);
-    k_assemble<C><<<(unsigned)a.ne, AsmSmem<C>::NTH, AsmSmem<C>::bytes, s>>>(a, ctx->T);
+    fp64_pointwise<C>(sm, a, ctx->T, ctx->ph, s);
+    fp64_assemble<C>(sm, a, ctx->T, s);
     if (int rc_b = boundary_patch(ctx, a, HDG_PREC_FP64, s)) return rc_b;
-    k_condense<C><<<(unsigned)a.ne, CondSmem<C>::NTH, CondSmem<C>::bytes, s>>>(a);
+    fp64_condense<C>(sm, a, s);
   }
   HDG_CK(cudaGetLastError());
   return HDG_OK;

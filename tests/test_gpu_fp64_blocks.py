@@ -36,3 +36,25 @@ def test_ragged_blocks_match_oracle(case):
         scale = max(np.abs(ref["Rl"][nq:]).max(), np.abs(ref["Rt"]).max(), np.abs(hist[e]).max(), 1.0)
         assert np.abs(R[e, :nv] - ref["Rl"][nq:]).max() <= 1e-12 * scale
         assert np.abs(R[e, nv:] - ref["Rt"]).max() <= 1e-12 * scale
+
+
+@pytest.mark.parametrize("p", [3, 4])
+def test_elements_past_the_small_mesh_rule_match_oracle(p):
+    """2D meshes of more than 304 elements take the blocked kernels, smaller ones those for small elements: both sides of
+    the line give the oracle's blocks on sampled elements, at the same tolerance."""
+    for n in (12, 13):                                    # 288 and 338 triangles
+        case = Case(f"ns2d_p{p}", 2, n, p, 4.0, 0.5, 500.0, 0.71, "vortex")
+        prob, Q, V, Vh = oracle_setup(case)
+        gc = GpuCase(case)
+        hist = gc.history()
+        gc.assemble(hist)
+        assert int(gc.status.abs().sum()) == 0
+        i = gc.info
+        S, g, rec = (t.cpu().numpy() for t in (gc.S, gc.g, gc.recov))
+        for e in (0, 1, i["n_elem"] - 1):
+            he = prob.history_weak(e, [V[e] * (1 + 1e-3)], [case.mass_coef])
+            ref = prob.condense(e, Q[e], V[e], prob.gather_trace(Vh, e), case.mass_coef, he)
+            nv, nt = i["nv"], i["nt"]
+            assert rel_fro(S[e], ref["S"]) <= 1e-10
+            assert rel_fro(g[e], ref["g"]) <= 1e-10
+            assert rel_fro(rec[e, :nv * nt].reshape(nv, nt), ref["X"][Q[e].size:]) <= 1e-10

@@ -32,4 +32,6 @@ def test_ragged_tiles_and_uniform_far_field(case):
     for e in range(gc.info["n_elem"]):
         assert rel_fro(S[e], ref["S"][e]) <= 1e-10, e
         assert rel_fro(g[e], ref["g"][e]) <= 1e-10, e
-    assert (R == ref["R"]).all()
+    # the two forms' residuals may come from different kernels (small elements): FP64 rounding of the summed terms
+    scale = max(abs(ref["R"]).max(), float(hist.abs().max()), 1.0)
+    assert abs(R - ref["R"]).max() <= 1e-12 * scale
