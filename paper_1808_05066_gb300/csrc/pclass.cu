@@ -441,7 +441,7 @@ int pclass_index(int pk, int pt) {
 int assemble_condense_pclass(hdg_ctx* c, const double* V, const double* Vhat, const double* hist, double mass_coef,
                              double* S, double* g, double* recov, double* R, int32_t* status, cudaStream_t s) {
   PMix& pm = *c->pm;
-  if (!pm.attr_set) {  // per context, hence per device
+  if (!pm.attr_set) {
     int optin = 0, per_sm = 0;
     cudaFuncAttributes fa{};
     HDG_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
@@ -450,7 +450,10 @@ int assemble_condense_pclass(hdg_ctx* c, const double* V, const double* Vhat, co
       set_error("assemble_condense: the element classes need more shared memory than the device has");
       return HDG_ERR_UNSUPPORTED;
     }
-    HDG_CK(cudaFuncSetAttribute(k_pclass_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pm.smem_bytes));
+    // the limit belongs to the kernel and the device, not to this context: always the most there is, as another
+    // context's classes may need more than this one's
+    HDG_CK(cudaFuncSetAttribute(k_pclass_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                optin - (int)fa.sharedSizeBytes));
     HDG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pclass_fused, kThreads, pm.smem_bytes));
     pm.ctas = (int)std::min<int64_t>(c->E, (int64_t)std::max(1, per_sm) * (c->num_sms > 0 ? c->num_sms : 152));
     pm.attr_set = true;
