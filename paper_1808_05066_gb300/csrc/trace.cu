@@ -851,8 +851,9 @@ int launch_trace_matvec(hdg_ctx* ctx, const double* S, const double* x, double* 
 // (2D p = 4, 8,192 elements) 8.5 against 7.7.
 // The ring's slots per warp, as many of up to four as fit into an SM's shared memory (0: elements that take the other form).
 constexpr int kMvRingNT = 96;
+constexpr size_t kMvRingSmem = (size_t)222 * 1024;  // all warps' rings
 static int matvec_ring_slots(const hdg_ctx* ctx, size_t* smem) {
-  const size_t slot = sizeof(df2) * kMvRows * ctx->NT, xs = sizeof(df2) * ctx->NT, room = (size_t)222 * 1024 / kMvWarps;
+  const size_t slot = sizeof(df2) * kMvRows * ctx->NT, xs = sizeof(df2) * ctx->NT, room = kMvRingSmem / kMvWarps;
   const int n = room < xs ? 0 : (int)std::min<size_t>(kMvMaxSlots, (room - xs) / slot);
   *smem = kMvWarps * (n * slot + xs);
   return ctx->NT >= kMvRingNT && n >= 2 && ctx->NT % 2 == 0 ? n : 0;  // copies start on 16 bytes
@@ -862,8 +863,9 @@ static int matvec_ring_slots(const hdg_ctx* ctx, size_t* smem) {
 // these steps may be captured)
 static int prepare_matvec_df(hdg_ctx* ctx) {
   size_t smem;
-  if (!ctx->attr_matvec && matvec_ring_slots(ctx, &smem)) {  // per context, hence per device
-    HDG_CK(cudaFuncSetAttribute(k_elem_matvec_ring, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (!ctx->attr_matvec && matvec_ring_slots(ctx, &smem)) {
+    // the limit belongs to the kernel and the device: the same for every context, whatever its own size
+    HDG_CK(cudaFuncSetAttribute(k_elem_matvec_ring, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMvRingSmem));
     if (!ctx->num_sms) HDG_CK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
     if (!ctx->d_mv_err) {
       HDG_CK(cudaMalloc(&ctx->d_mv_err, sizeof(int)));

@@ -49,3 +49,23 @@ def test_mixed_degree_assembly():
     small.assemble()
     for k, v in large.assemble().items():
         assert large.torch.equal(v, first[k]), k
+
+
+def _solve(flow):
+    """GMRES into a new output buffer: a recorded cycle refers to its buffers and is recorded again."""
+    x = flow.torch.empty_like(flow.Vhat)
+    it, res = flow.hdg.hdg_trace_solve(flow.ctx.handle, flow.out["S"], flow.out["g"], x, flow.hdg.HDG_SOLVER_GMRES,
+                                       1e-10, 600)
+    assert it > 1 and res <= 1e-10
+    return x
+
+
+def test_trace_products():
+    large, small = Flow(2, 3), Flow(2, 2)   # rings of 200 and 120 columns
+    for f in (large, small):
+        f.assemble()
+    xs = [_solve(f) for f in (large, small, large)]
+    torch = large.torch
+    assert float(torch.linalg.norm(xs[2] - xs[0])) <= 1e-6 * float(torch.linalg.norm(xs[0]))
+    c, r = large.hdg.hdg_ctx_trace_cycles(large.ctx.handle)
+    assert c == r                           # every cycle a graph replay: nothing was refused while recording
