@@ -384,7 +384,10 @@ int pm_face_factor(hdg_ctx* c, const double* S, double* pc, cudaStream_t s) {
   const int B = c->pm->nfn_max * M5;
   const size_t sm = 2 * sizeof(double) * B * B;
   if (!c->pm->attr_face) {
-    HDG_CK(cudaFuncSetAttribute(k_pm_face_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    // the limit belongs to the kernel and the device: the widest face's (degree 4), whatever this context's own
+    constexpr int kWidest = 15 * M5;
+    HDG_CK(cudaFuncSetAttribute(k_pm_face_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                2 * (int)sizeof(double) * kWidest * kWidest));
     c->pm->attr_face = true;
   }
   k_pm_face_factor<<<(unsigned)c->F, 128, sm, s>>>(pmix_dev(c), S, pc);

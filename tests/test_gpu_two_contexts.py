@@ -69,3 +69,12 @@ def test_trace_products():
     assert float(torch.linalg.norm(xs[2] - xs[0])) <= 1e-6 * float(torch.linalg.norm(xs[0]))
     c, r = large.hdg.hdg_ctx_trace_cycles(large.ctx.handle)
     assert c == r                           # every cycle a graph replay: nothing was refused while recording
+
+
+def test_mixed_degree_preconditioner():
+    large, small = Flow(2, 0, (4, 1, 3, 2, 4, 3)), Flow(2, 0, (1, 2, 2, 1, 1, 2))   # faces of 75 and 30 unknowns
+    for f in (large, small):
+        f.assemble()
+    xs = [_solve(f) for f in (large, small, large)]
+    torch = large.torch
+    assert float(torch.linalg.norm(xs[2] - xs[0])) <= 1e-6 * float(torch.linalg.norm(xs[0]))
