@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
         if (chunk != cur) {
           cur = chunk;
           const int E = er[cur * 128];
-          rs = E > 1000 ? __int_as_float(0x7fffffff) : oz_pow2(E);  // NaN: an entry that is no finite number
+          rs = E > 127 ? __int_as_float(0x7fffffff) : oz_pow2(E);  // NaN: an entry beyond the float range
         }
         const int kind = (job >> T5_KIND) & 3;
         unsigned char* od = kind == T5_COL_FI ? out[2] : out[3];
