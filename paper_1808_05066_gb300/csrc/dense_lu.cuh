@@ -430,6 +430,15 @@ __global__ void __cluster_dims__(kLuCluster, 1, 1) __launch_bounds__(256)
           if (lane == t) v = qc;
           if (lane < t) v -= T[lane][t] * xt;
         }
+        // again with divisions if that left something that is no finite number (an infinite or subnormal d)
+        if (__any_sync(0xffffffffu, (__double2hiint(v) & 0x7ff00000) == 0x7ff00000)) {
+          v = vb[b][lane];
+          for (int t = m - 1; t >= 0; --t) {
+            const double xt = __shfl_sync(0xffffffffu, v / d, t);
+            if (lane == t) v = xt;
+            if (lane < t) v -= T[lane][t] * xt;
+          }
+        }
       }
       if (lane < m) xs[i0 + lane] = v;
     }
