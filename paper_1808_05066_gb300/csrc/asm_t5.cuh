@@ -33,6 +33,12 @@
 //
 // Two row programs: pairs (i, l) with a viscous part (i, l > 0), and those without, which need the value
 // operators only (elsewhere their blocks are zero).
+//
+// A mesh with fewer tiles than half the SMs would leave the chip idle while one CTA walks a tile's whole job list, so
+// the planes are dealt by test node to several parts, each with a job list of its own (all columns of a plane
+// have the same test node), and a tile is taken by one CTA per part. A plane's additions keep their order: the blocks are
+// the same bit for bit. 48 tetrahedra, p = 3 (10 tiles): 0.14 ms in ten parts, 0.69 in one; the whole call 1.02 ms, 1.63
+// in one part; 128 triangles, p = 3: 0.29 ms, 0.34.
 #pragma once
 #include "assemble_fp64.cuh"
 #include "condense_t5.cuh"
@@ -69,16 +75,17 @@ struct T5Col {
 
 struct T5Prog {  // device pointers
   const int* jobs;
-  T5Col* cols;           // [njob + 2][32] (two empty groups behind the last)
+  T5Col* cols;           // [jobs of all parts + 2][32] (two empty groups behind the last)
   const unsigned char* W;
   const int* pairs;      // [rpe] i << 8 | l
   const T5Entry* ent;    // [nchunk][128]
   const int* cstep;      // [nchunk + 1] first step of each chunk
-  const int* wstep;      // [njob] first step of each job in W
-  const int* zero;       // [nzero] entries that vanish for these pairs
-  const unsigned char* T;  // slices of the rows [tile][steps][6][4 KB]
+  const int* wstep;      // [jobs] first step of each job in W
+  const int* zero;       // entries that vanish for these pairs
+  const int2* part;      // [nparts + 1] first job and first zero entry of each part
+  unsigned char* T;        // slices of the rows [tile][steps][6][4 KB]
   int* erow;             // [tile][nchunk][128]
-  int njob, nchunk, rpe, ept, ntile, nsteps, nzero;
+  int nchunk, rpe, ept, ntile, nsteps;
 };
 
 // Integer slices of a double: F = v 2^(48 - E) rounded to an integer (|v| < 2^E), split into balanced base-256
@@ -128,15 +135,30 @@ HDG_DEVI void t5_put8(unsigned char* blk, uint32_t stride, uint32_t off, const d
 }
 
 // ------------------------------------------------------------------------------------
-// k_t5_rows: row exponents and slices of one (tile, chunk) from the FP64 point tensors. The maximum and
-// the slices read the values twice (the second time from L1).
+// k_t5_rows: the two passes over the FP64 point tensors. A block forms the row exponents and slices of one (chunk, tile),
+// program 0's before program 1's (the maximum and the slices read the values twice, the second time from L1), or,
+// behind those, one element's residuals R_v and R_t in FP64. One launch: each part alone waits for its own latency
+// on a small mesh (128 triangles, p = 3: 57 us in three launches, 32 in one).
 // ------------------------------------------------------------------------------------
 template <class C>
-__global__ void __launch_bounds__(256) k_t5_rows(AssembleArgs a, T5Prog P, unsigned char* T) {
+__global__ void __launch_bounds__(256) k_t5_rows(AssembleArgs a, DevTables Tb, T5Prog P0, T5Prog P1) {
   constexpr int D = C::D, M = C::M, MV = M - 1, NG = C::NG, NQ = C::NF * C::NGF;
+  const int tid = threadIdx.x, n0 = P0.ntile * P0.nchunk, n1 = P1.ntile * P1.nchunk;
+  if ((int)blockIdx.x >= n0 + n1) {
+    __shared__ ElemTables<D> E;
+    const int64_t le = blockIdx.x - n0 - n1, e = a.e0 + le;
+    if (tid == 0) uniform_tables<C>(Tb, E);
+    __syncthreads();
+    double* R = a.R + e * (int64_t)(C::NV + C::NT);
+    element_residual<D, 256>(UniformDims<C>(), E, a.ptv + le * NG * C::PT_VOL, a.ptf + le * NQ * C::PT_FACE,
+                             a.hist ? a.hist + e * C::NV : nullptr, R, R + C::NV);
+    return;
+  }
   __shared__ T5Entry ent[128];
   __shared__ unsigned long long mx[128];
-  const int tile = blockIdx.x, ch = blockIdx.y, tid = threadIdx.x;
+  const bool p0 = (int)blockIdx.x < n0;
+  const T5Prog& P = p0 ? P0 : P1;
+  const int at = p0 ? blockIdx.x : blockIdx.x - n0, tile = at % P.ntile, ch = at / P.ntile;
   const int s0 = P.cstep[ch], nk = P.cstep[ch + 1] - s0;
   for (int t = tid; t < 128; t += 256) {
     ent[t] = P.ent[ch * 128 + t];
@@ -183,7 +205,7 @@ __global__ void __launch_bounds__(256) k_t5_rows(AssembleArgs a, T5Prog P, unsig
   __syncthreads();
   const int E = t5_exponent(__longlong_as_double((long long)mx[row]));
   if (tid < 128) P.erow[((int64_t)tile * P.nchunk + ch) * 128 + row] = E;
-  unsigned char* dst = T + ((int64_t)tile * P.nsteps + s0) * kT5Slices * kT5ATile;
+  unsigned char* dst = P.T + ((int64_t)tile * P.nsteps + s0) * kT5Slices * kT5ATile;
   for (int kg = tid >> 7; kg < 2 * nk; kg += 2) {
     double v[8];
     load8(kg, v);
@@ -305,14 +327,14 @@ constexpr size_t kT5Smem = (size_t)kT5Steps * kT5Slices * kT5ATile + (size_t)kT5
                            kT5Epi * kT5Q * sizeof(T5Col) + sizeof(int) * kT5MaxJobs;
 
 // ------------------------------------------------------------------------------------
-// k_asm_t5: tiles [0, P0.ntile) of program 0, then those of program 1. planes: [grid][nplane + 1][128]
-// (the last one takes the empty columns).
+// k_asm_t5: tiles [0, P0.ntile) of program 0, then those of program 1; CTA b takes part b % nparts of every
+// (gridDim.x / nparts)-th one. planes: [grid][nplane + 1][128] (the last one takes the empty columns).
 // Every wait is bounded; one that gives up sets s_fail, all roles then leave, the copies and MMAs in
 // flight drain, and the tile's elements get HDG_STATUS_TIMEOUT.
 // ------------------------------------------------------------------------------------
 template <class C>
 __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog P0, T5Prog P1, df2* planes,
-                                                          int nplane) {
+                                                          int nplane, int nparts) {
   constexpr int NV = C::NV, NT = C::NT;
   constexpr uint32_t ASTEP = kT5Slices * kT5ATile, WSTEP = kT5Slices * kT5BTile;
   extern __shared__ __align__(128) unsigned char smem_t5[];
@@ -331,6 +353,14 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
   __shared__ uint32_t s_tmem;
   __shared__ volatile int s_fail;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ int4 s_part[2];  // this part of both programs: first job, jobs, first zero entry, end of its zero entries
+  const int first = blockIdx.x / nparts, stride = gridDim.x / nparts;
+  if (tid < 2) {
+    const T5Prog& P = tid ? P1 : P0;
+    const int2* pt = P.part + blockIdx.x % nparts;
+    s_part[tid] = P.ntile ? make_int4(pt[0].x, pt[1].x - pt[0].x, pt[0].y, pt[1].y) : make_int4(0, 0, 0, 0);
+  }
+  __syncthreads();
   if (tid == 0) {
     s_fail = 0;
     for (int i = 0; i < 2 * kT5Steps + 2 * kT5Ring; ++i) mbar_init(bars + i, 1);
@@ -341,8 +371,8 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
     mbar_init(drain, 1);
     fence_mbar_init();
   }
-  for (int t = tid; t < P0.njob; t += kT5Threads) sjobs[t] = P0.jobs[t];
-  for (int t = tid; t < P1.njob; t += kT5Threads) sjobs[P0.njob + t] = P1.jobs[t];
+  for (int t = tid; t < s_part[0].y; t += kT5Threads) sjobs[t] = P0.jobs[s_part[0].x + t];
+  for (int t = tid; t < s_part[1].y; t += kT5Threads) sjobs[s_part[0].y + t] = P1.jobs[s_part[1].x + t];
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512)
                  : "memory");
@@ -360,14 +390,15 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
       int w = 0, w_par = 1, nw = 0;
       uint32_t a_out = 0;              // per slot: loads issued, modulo 2 (for the drain)
       bool ok = true;
-      for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
+      for (int t = first; t < ntile && ok; t += stride) {
         const bool p0 = t < P0.ntile;
         const T5Prog& P = p0 ? P0 : P1;
-        const int* jobs = sjobs + (p0 ? 0 : P0.njob);
+        const int* jobs = sjobs + (p0 ? 0 : s_part[0].y);
+        const int njob = s_part[p0 ? 0 : 1].y;
         const unsigned char* Ts = P.T + (int64_t)(p0 ? t : t - P0.ntile) * P.nsteps * ASTEP;
-        const unsigned char* W = P.W;
+        const unsigned char* W = P.W + (int64_t)P.wstep[s_part[p0 ? 0 : 1].x] * WSTEP;
         int cur = -1;
-        for (int j = 0; j < P.njob && ok; ++j) {
+        for (int j = 0; j < njob && ok; ++j) {
           const int job = jobs[j], chunk = (job >> 8) & 255;
           if (chunk != cur) {
             cur = chunk;
@@ -414,11 +445,12 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
       int w = 0, w_par = 0, buf = 0, e_par = 1;
       bool ok = true;
       const uint64_t adesc0 = umma_desc(smem_u32(As), 128, 256), wdesc0 = umma_desc(smem_u32(Ws), 128, 256);
-      for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
+      for (int t = first; t < ntile && ok; t += stride) {
         const bool p0 = t < P0.ntile;
         const T5Prog& P = p0 ? P0 : P1;
-        const int* jobs = sjobs + (p0 ? 0 : P0.njob);
-        for (int j = 0; j < P.njob && ok; ++j) {
+        const int* jobs = sjobs + (p0 ? 0 : s_part[0].y);
+        const int njob = s_part[p0 ? 0 : 1].y;
+        for (int j = 0; j < njob && ok; ++j) {
           const int job = jobs[j], used = job & 255;
           ok = t5_wait(acc_empty + buf, e_par) && !s_fail;  // the first use of each buffer passes at once
           if (!ok) break;
@@ -481,11 +513,12 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
     int4* sc = scols + warp * kT5Q;
     int f_par = 0, turn = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
+    for (int t = first; t < ntile && ok; t += stride) {
       const bool p0 = t < P0.ntile;
       const T5Prog& P = p0 ? P0 : P1;
-      const int* jobs = sjobs + (p0 ? 0 : P0.njob);
-      const int tile = p0 ? t : t - P0.ntile, njob = P.njob, el = row / P.rpe;
+      const int* jobs = sjobs + (p0 ? 0 : s_part[0].y);
+      const int4 mine = s_part[p0 ? 0 : 1];
+      const int tile = p0 ? t : t - P0.ntile, njob = mine.y, el = row / P.rpe;
       const int64_t le = (int64_t)tile * P.ept + el, e = a.e0 + le;
       const bool live = el < P.ept && le < a.ne;
       const int pr = live ? P.pairs[row % P.rpe] : 0, i = pr >> 8, l = pr & 255;
@@ -494,7 +527,8 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
       out[1] = reinterpret_cast<unsigned char*>(a.recov + e * (int64_t)(NV * NT + NV) + i * NT + l);
       out[2] = reinterpret_cast<unsigned char*>(a.Cp + le * NT * NV + i * NV + l);
       out[3] = reinterpret_cast<unsigned char*>(a.S + e * (int64_t)NT * NT + i * NT + l);
-      const int4* ct = reinterpret_cast<const int4*>(P.cols) + kT5Q * part + (lane & (kT5Q - 1));
+      const int4* ct = reinterpret_cast<const int4*>(P.cols) + mine.x * kT5Cols + kT5Q * part +
+                       (lane & (kT5Q - 1));
       const int* er = P.erow + (int64_t)tile * P.nchunk * 128 + row;
       auto load_y = [&](int job, const int4& cc, df2 (&dst)[kT5Q]) {
         if (job & T5_FIRST) return;
@@ -584,7 +618,7 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
         s_fail = 1;
         break;
       }
-      for (int z = part; z < P.nzero; z += kT5Epi / 4) {  // zero[]: array << 28 | byte offset / 8
+      for (int z = s_part[p0 ? 0 : 1].z + part; z < s_part[p0 ? 0 : 1].w; z += kT5Epi / 4) {  // zero[]: array << 28 | byte offset / 8
         const int w = P.zero[z], arr = w >> 28;
         unsigned char* p = arr == 0 ? out[0] : arr == 1 ? out[1] : arr == 2 ? out[2] : out[3];
         if (live) reinterpret_cast<df2*>(p)[w & 0xfffffff] = df2{0.f, 0.f};
@@ -593,7 +627,7 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
   }
   __syncthreads();
   if (s_fail)  // every element of this CTA's tiles is recomputed (or reported)
-    for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
+    for (int t = first; t < ntile; t += stride) {
       const T5Prog& P = t < P0.ntile ? P0 : P1;
       const int64_t l0 = (int64_t)(t < P0.ntile ? t : t - P0.ntile) * P.ept;
       for (int x = tid; x < P.ept; x += kT5Threads)
@@ -603,19 +637,6 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
   __syncthreads();
   tc_fence_after();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-}
-
-// R_v and R_t (FP64 from the point tensors), one CTA per element
-template <class C>
-__global__ void __launch_bounds__(128) k_residual(AssembleArgs a, DevTables T) {
-  __shared__ ElemTables<C::D> E;
-  const int64_t le = blockIdx.x, e = a.e0 + le;
-  if (threadIdx.x == 0) uniform_tables<C>(T, E);
-  __syncthreads();
-  const UniformDims<C> d;
-  double* R = a.R + e * (int64_t)(C::NV + C::NT);
-  element_residual<C::D, 128>(d, E, a.ptv + le * C::NG * C::PT_VOL, a.ptf + le * C::NF * C::NGF * C::PT_FACE,
-                              a.hist ? a.hist + e * C::NV : nullptr, R, R + C::NV);
 }
 
 }  // namespace hdg

@@ -16,13 +16,14 @@ namespace hdg {
 namespace {
 
 constexpr int kSlices = 6;  // exact bf16 slices per operand in every tensor-core product
+constexpr int64_t kMixedChunk = 8192;  // elements per chunk, unless their scratch is too large
 
 }  // namespace
 
 // The assembly's constant operand and its schedule (asm_t5.cuh), built on the first mixed call of a context.
 struct T5Plan {
   T5Prog prog[2] = {};  // rows with a viscous part, rows without
-  int nplane = 0;
+  int nplane = 0, nparts = 1;
   df2* planes = nullptr;
   std::vector<void*> bufs;
   ~T5Plan() {
@@ -42,10 +43,10 @@ int t5_upload(T5Plan& pl, const std::vector<T>& v, T** out) {
   return HDG_OK;
 }
 
-// One row program: its entries of k in chunks of at most 128, and per chunk the groups of up to 32
+// One row program: its entries of k in chunks of at most 128, and per part and chunk the groups of up to 32
 // columns that use the same steps of 16 entries.
 template <class C>
-int t5_program(hdg_ctx* ctx, T5Plan& pl, bool viscous, T5Prog& P, cudaStream_t s) {
+int t5_program(hdg_ctx* ctx, T5Plan& pl, bool viscous, T5Prog& P, int* jobs_of_part, cudaStream_t s) {
   constexpr int D = C::D, M = C::M, NP = C::NP, NFN = C::NFN, NF = C::NF, NG = C::NG, NGF = C::NGF, NV = C::NV,
                 NT = C::NT, NTN = NF * NFN;
   const RefElement& ref = ctx->mesh->m.ref;
@@ -101,7 +102,7 @@ int t5_program(hdg_ctx* ctx, T5Plan& pl, bool viscous, T5Prog& P, cudaStream_t s
   // columns
   struct Col {
     T5ColDesc d;
-    int plane, direct;
+    int node, plane, direct;  // node: the plane's test node
   };
   std::vector<char> on_face(NF * NP, 0);
   for (int f = 0; f < NF; ++f)
@@ -112,23 +113,23 @@ int t5_program(hdg_ctx* ctx, T5Plan& pl, bool viscous, T5Prog& P, cudaStream_t s
   for (int a = 0; a < NP; ++a) {
     for (int j = 0; j < NP; ++j) {
       fin[a * NP + j] = a * M * NV + j * M;
-      all.push_back({{T5_COL_A, 0, (short)a, (short)j, 0, 0}, a * NP + j, -1});
+      all.push_back({{T5_COL_A, 0, (short)a, (short)j, 0, 0}, a, a * NP + j, -1});
     }
     for (int f = 0; f < NF; ++f)
       for (int c = 0; c < NFN; ++c) {
         const int p = NP * NP + a * NTN + f * NFN + c;
         fin[p] = 1 << 28 | (a * M * NT + (f * NFN + c) * M);
-        all.push_back({{T5_COL_B, (short)f, (short)a, (short)c, 0, 0}, p, -1});
+        all.push_back({{T5_COL_B, (short)f, (short)a, (short)c, 0, 0}, a, p, -1});
       }
   }
   for (int f = 0; f < NF; ++f)
     for (int c = 0; c < NFN; ++c) {
       const int node = ref.face_nodes[f][c], row = (f * NFN + c) * M;
       for (int j = 0; j < NP; ++j)
-        all.push_back({{T5_COL_FI, (short)f, (short)c, (short)j, 0, 0}, node * NP + j, 2 << 28 | (row * NV + j * M)});
+        all.push_back({{T5_COL_FI, (short)f, (short)c, (short)j, 0, 0}, node, node * NP + j, 2 << 28 | (row * NV + j * M)});
       for (int f2 = 0; f2 < NF; ++f2)
         for (int c2 = 0; c2 < NFN; ++c2)
-          all.push_back({{T5_COL_FT, (short)f, (short)c, (short)c2, (short)f2, 0},
+          all.push_back({{T5_COL_FT, (short)f, (short)c, (short)c2, (short)f2, 0}, node,
                          NP * NP + node * NTN + f2 * NFN + c2, 3 << 28 | (row * NT + (f2 * NFN + c2) * M)});
     }
   auto uses = [&](const T5ColDesc& d, const T5Entry& e) {
@@ -157,73 +158,90 @@ int t5_program(hdg_ctx* ctx, T5Plan& pl, bool viscous, T5Prog& P, cudaStream_t s
         ++left[all[k].plane];
       }
     }
+  // the test nodes' parts: the heaviest first, each to the lightest part (a column costs its steps and its additions)
+  std::vector<int> weight(NP, 0), order(NP), load(pl.nparts, 0), part_of(NP);
+  for (int ch = 0; ch < P.nchunk; ++ch)
+    for (size_t k = 0; k < all.size(); ++k)
+      if (masks[ch][k]) weight[all[k].node] += __builtin_popcount(masks[ch][k]) + 2;
+  for (int a = 0; a < NP; ++a) order[a] = a;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return weight[a] > weight[b]; });
+  for (int a : order) {
+    part_of[a] = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    load[part_of[a]] += weight[a];
+  }
   const T5Col none = {nplane * 128 * (int)sizeof(df2), -1, 0.f, -1};
-  std::vector<int> jobs, wstep;
+  std::vector<int> jobs, wstep, zero;  // zero: entries that vanish for these pairs
+  std::vector<int2> parts;
   std::vector<T5Col> cols;
   std::vector<T5ColDesc> desc;
   int wsteps = 0;
-  std::set<int> before;  // planes of the job before
-  for (int ch = 0; ch < P.nchunk; ++ch) {
-    std::map<std::array<int, 4>, std::vector<int>> groups;  // (not first, last, kind, steps)
-    for (size_t k = 0; k < all.size(); ++k)
-      if (masks[ch][k]) {
-        const int p = all[k].plane;
-        groups[{seen[p] ? 1 : 0, --left[p] ? 0 : 1, all[k].d.kind, masks[ch][k]}].push_back((int)k);
-        ++seen[p];
-      }
-    for (auto& gr : groups) {
-      std::vector<int> rest = gr.second;
-      while (!rest.empty()) {
-        int job = gr.first[3] | ch << 8 | (gr.first[0] ? 0 : T5_FIRST) | (gr.first[1] ? T5_LAST : 0) |
-                  gr.first[2] << T5_KIND;
-        wstep.push_back(wsteps);
-        for (int m = gr.first[3]; m; m &= m - 1) ++wsteps;
-        cols.resize((jobs.size() + 1) * kT5Cols, none);
-        desc.resize((jobs.size() + 1) * kT5Cols, {T5_COL_NONE, 0, 0, 0, 0, 0});
-        int fill[4] = {0, 0, 0, 0};
-        std::set<int> taken;
-        std::vector<int> later;
-        for (int k : rest) {
-          const Col& c = all[k];
-          const int h = quarter(c.plane);
-          if (fill[h] == kT5Q || taken.count(c.plane)) {
-            later.push_back(k);
-            continue;
-          }
-          taken.insert(c.plane);
-          if (before.count(c.plane)) job |= T5_HAZARD;
-          const size_t at = jobs.size() * kT5Cols + h * kT5Q + fill[h]++;
-          cols[at] = {c.plane * 128 * (int)sizeof(df2), c.direct < 0 ? -1 : (c.direct & 0xfffffff) * 8, 0.f,
-                      (fin[c.plane] & 0xfffffff) * 8};
-          desc[at] = c.d;
+  for (int part = 0; part < pl.nparts; ++part) {
+    parts.push_back(make_int2((int)jobs.size(), (int)zero.size()));
+    std::set<int> before;  // planes of the job before
+    for (int ch = 0; ch < P.nchunk; ++ch) {
+      std::map<std::array<int, 4>, std::vector<int>> groups;  // (not first, last, kind, steps)
+      for (size_t k = 0; k < all.size(); ++k)
+        if (masks[ch][k] && part_of[all[k].node] == part) {
+          const int p = all[k].plane;
+          groups[{seen[p] ? 1 : 0, --left[p] ? 0 : 1, all[k].d.kind, masks[ch][k]}].push_back((int)k);
+          ++seen[p];
         }
-        rest.swap(later);
-        before.swap(taken);
-        jobs.push_back(job);
+      if (groups.empty()) continue;
+      for (auto& gr : groups) {
+        std::vector<int> rest = gr.second;
+        while (!rest.empty()) {
+          int job = gr.first[3] | ch << 8 | (gr.first[0] ? 0 : T5_FIRST) | (gr.first[1] ? T5_LAST : 0) |
+                    gr.first[2] << T5_KIND;
+          wstep.push_back(wsteps);
+          for (int m = gr.first[3]; m; m &= m - 1) ++wsteps;
+          cols.resize((jobs.size() + 1) * kT5Cols, none);
+          desc.resize((jobs.size() + 1) * kT5Cols, {T5_COL_NONE, 0, 0, 0, 0, 0});
+          int fill[4] = {0, 0, 0, 0};
+          std::set<int> taken;
+          std::vector<int> later;
+          for (int k : rest) {
+            const Col& c = all[k];
+            const int h = quarter(c.plane);
+            if (fill[h] == kT5Q || taken.count(c.plane)) {
+              later.push_back(k);
+              continue;
+            }
+            taken.insert(c.plane);
+            if (before.count(c.plane)) job |= T5_HAZARD;
+            const size_t at = jobs.size() * kT5Cols + h * kT5Q + fill[h]++;
+            cols[at] = {c.plane * 128 * (int)sizeof(df2), c.direct < 0 ? -1 : (c.direct & 0xfffffff) * 8, 0.f,
+                        (fin[c.plane] & 0xfffffff) * 8};
+            desc[at] = c.d;
+          }
+          rest.swap(later);
+          before.swap(taken);
+          jobs.push_back(job);
+        }
       }
+      jobs.back() |= T5_CLOSES;
     }
-    jobs.back() |= T5_CLOSES;
+    for (int p = 0; p < nplane; ++p)
+      if (!seen[p] && part_of[p < NP * NP ? p / NP : (p - NP * NP) / NTN] == part) zero.push_back(fin[p]);
+    for (size_t k = 0; k < all.size(); ++k)
+      if (!written[k] && all[k].direct >= 0 && part_of[all[k].node] == part) zero.push_back(all[k].direct);
+    jobs_of_part[part] += (int)jobs.size() - parts[part].x;
   }
-  std::vector<int> zero;  // entries that vanish for these pairs
-  for (int p = 0; p < nplane; ++p)
-    if (!seen[p]) zero.push_back(fin[p]);
-  for (size_t k = 0; k < all.size(); ++k)
-    if (!written[k] && all[k].direct >= 0) zero.push_back(all[k].direct);
+  parts.push_back(make_int2((int)jobs.size(), (int)zero.size()));
   for (int k = 0; k < 2 * kT5Cols; ++k) cols.push_back(none);
-  P.njob = (int)jobs.size();
-  P.nzero = (int)zero.size();
   pl.nplane = nplane;
   int *dj, *dc, *dp, *dws, *dz;
+  int2* dpart;
   T5Entry* de;
   T5ColDesc* dd;
   unsigned char* dw;
   int rc;
   if ((rc = t5_upload(pl, jobs, &dj)) || (rc = t5_upload(pl, cols, &P.cols)) || (rc = t5_upload(pl, desc, &dd)) ||
       (rc = t5_upload(pl, ent, &de)) || (rc = t5_upload(pl, cstep, &dc)) || (rc = t5_upload(pl, pairs, &dp)) ||
-      (rc = t5_upload(pl, wstep, &dws)) || (rc = t5_upload(pl, zero, &dz)))
+      (rc = t5_upload(pl, wstep, &dws)) || (rc = t5_upload(pl, zero, &dz)) || (rc = t5_upload(pl, parts, &dpart)))
     return rc;
   P.wstep = dws;
   P.zero = dz;
+  P.part = dpart;
   HDG_CK(cudaMalloc(&dw, (size_t)wsteps * kT5Slices * kT5BTile));
   pl.bufs.push_back(dw);
   P.jobs = dj;
@@ -231,17 +249,32 @@ int t5_program(hdg_ctx* ctx, T5Plan& pl, bool viscous, T5Prog& P, cudaStream_t s
   P.cstep = dc;
   P.pairs = dp;
   P.W = dw;
-  k_t5_weights<C><<<P.njob, 256, 0, s>>>(ctx->T, P, dd, dw);
+  k_t5_weights<C><<<(unsigned)jobs.size(), 256, 0, s>>>(ctx->T, P, dd, dw);
   HDG_CK(cudaGetLastError());
   return HDG_OK;
+}
+
+// Parts of a tile's planes for a chunk of n elements: as many as there are idle SMs per tile, but no more than leave
+// every part the same number of test nodes (20 nodes in 15 parts take as long as in 10).
+template <class C>
+int t5_parts(int64_t n, int num_sms) {
+  constexpr int M = C::M, MV = M - 1, VP = C::VISC ? MV * MV : 0;  // pairs with a viscous part
+  const auto tiles = [&](int pairs) { return pairs ? (n + 128 / pairs - 1) / (128 / pairs) : 0; };
+  const int64_t room = num_sms / (tiles(VP) + tiles(M * M - VP));
+  if (room < 2) return 1;
+  const int64_t nodes = (C::NP + room - 1) / room;  // of a part
+  return (int)((C::NP + nodes - 1) / nodes);
 }
 
 template <class C>
 int t5_plan(hdg_ctx* ctx, cudaStream_t s) {
   if (ctx->t5_plan) return HDG_OK;
   auto* pl = new T5Plan();
+  pl->nparts = t5_parts<C>(ctx->chunk ? ctx->chunk : std::min<int64_t>(ctx->E, kMixedChunk), ctx->num_sms);
+  std::vector<int> jobs(pl->nparts, 0);
   int rc = HDG_OK;
-  if ((rc = t5_program<C>(ctx, *pl, true, pl->prog[0], s)) || (rc = t5_program<C>(ctx, *pl, false, pl->prog[1], s))) {
+  if ((rc = t5_program<C>(ctx, *pl, true, pl->prog[0], jobs.data(), s)) ||
+      (rc = t5_program<C>(ctx, *pl, false, pl->prog[1], jobs.data(), s))) {
     delete pl;
     return rc;
   }
@@ -250,7 +283,7 @@ int t5_plan(hdg_ctx* ctx, cudaStream_t s) {
     return cuda_fail(cudaGetLastError(), "cudaMalloc (assembly planes)");
   }
   pl->bufs.push_back(pl->planes);
-  if (pl->prog[0].njob + pl->prog[1].njob > kT5MaxJobs) {
+  if (*std::max_element(jobs.begin(), jobs.end()) > kT5MaxJobs) {
     delete pl;
     set_error("assemble_condense: the assembly's schedule is longer than its table");
     return HDG_ERR_UNSUPPORTED;
@@ -275,13 +308,12 @@ template <class C>
 void run_asm_t5(hdg_ctx* ctx, const T5Plan& pl, const T5Prog (&pr)[2], const AssembleArgs& a, cudaStream_t s) {
   {
     LaunchScope ls(ctx, HDG_KERNEL_MIXED_OPERATORS, s);
-    for (const T5Prog& P : pr)
-      if (P.ntile)
-        k_t5_rows<C><<<dim3((unsigned)P.ntile, (unsigned)P.nchunk), 256, 0, s>>>(a, P, const_cast<unsigned char*>(P.T));
+    const int64_t blocks = (int64_t)pr[0].ntile * pr[0].nchunk + (int64_t)pr[1].ntile * pr[1].nchunk + a.ne;
+    k_t5_rows<C><<<(unsigned)blocks, 256, 0, s>>>(a, ctx->T, pr[0], pr[1]);
   }
   LaunchScope ls(ctx, HDG_KERNEL_MIXED_ASSEMBLE, s);
-  const int grid = std::min(ctx->num_sms, pr[0].ntile + pr[1].ntile);
-  k_asm_t5<C><<<grid, kT5Threads, kT5Smem, s>>>(a, pr[0], pr[1], pl.planes, pl.nplane);
+  const int grid = std::min(ctx->num_sms / pl.nparts, pr[0].ntile + pr[1].ntile) * pl.nparts;
+  k_asm_t5<C><<<grid, kT5Threads, kT5Smem, s>>>(a, pr[0], pr[1], pl.planes, pl.nplane, pl.nparts);
 }
 
 // One compiled shape of the condensation kernel, with the prep kernel that lays out its operands.
@@ -350,7 +382,7 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
   const size_t per_rows = t5_slice_bytes(pr[0], 1024) / 1024 + t5_slice_bytes(pr[1], 1024) / 1024;
   const size_t per = per_pt + slice_bytes + sizeof(float) * TC::prep_floats + per_rows;
   if (ctx->chunk == 0) {
-    int64_t ch = std::min<int64_t>(ctx->E, 8192);
+    int64_t ch = std::min<int64_t>(ctx->E, kMixedChunk);
     while (ch > 256 && per * ch > ((size_t)16 << 30)) ch /= 2;
     ctx->chunk = ch;
   }
@@ -424,10 +456,6 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
     {
       LaunchScope ls(ctx, HDG_KERNEL_POINTWISE, s);
       launch_pointwise<C>(a, ctx->T, ctx->ph, s);
-    }
-    {
-      LaunchScope ls(ctx, HDG_KERNEL_MIXED_OPERATORS, s);
-      k_residual<C><<<(unsigned)a.ne, 128, 0, s>>>(a, ctx->T);
     }
     for (T5Prog& P : pr) P.ntile = (int)t5_tiles(P, a.ne);
     if (ctx->cond_variant < 0 && a.ne >= 512) {
