@@ -372,7 +372,7 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
   T5Prog pr[2] = {pl.prog[0], pl.prog[1]};
   using TC = CondTC<C, 256, kSlices>;
   // the recomputation of flagged blocks may need more room for its point data
-  const bool sm = small::small_elements<C>(ctx->E);
+  const bool sm = small::small_elements<C>(ctx->E, ctx->num_sms);
   size_t vol, face, rvol, rface;
   point_doubles<C>(false, &vol, &face);
   point_doubles<C>(sm, &rvol, &rface);

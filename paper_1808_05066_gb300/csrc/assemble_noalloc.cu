@@ -57,7 +57,8 @@ template <class C>
 int run_noalloc(hdg_ctx* ctx, double* scratch, const double* V, const double* Vhat, const double* hist,
                 double mass_coef, double* S, double* g, double* recov, double* R, int32_t* status, cudaStream_t s) {
   using namespace hdg;
-  const bool sm = small::small_elements<C>(ctx->E);
+  if (!ctx->num_sms) HDG_CK(cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device));
+  const bool sm = small::small_elements<C>(ctx->E, ctx->num_sms);
   size_t vol, face;
   point_doubles<C>(sm, &vol, &face);
   const size_t per = vol + face + (size_t)C::NV * C::NV + (size_t)C::NT * C::NV;  // doubles per element

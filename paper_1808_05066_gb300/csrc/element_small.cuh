@@ -2,10 +2,17 @@
 // block. The kernels of element_fp64.cuh spread an element over register tiles and blocks; an element of a few
 // dozen unknowns does not fill those, and a mesh of fewer elements than the chip has room for waits for one
 // element's latency, which is shorter here.
-// small_elements() draws the line, both sides measured (assemble + condense, ms, here and there): 3D p = 1, 48,000 elements
-// 50.8, 58.6; 2D Euler p = 1 (51,200) 12.4, 12.5, p = 2 (32,768) 12.4, 13.9, p = 3 (18,432) 14.6, 15.3; 2D NS p = 2 (32,768)
-// 19.9, 21.6, but p = 3 (18,432) 23.1, 21.9 and p = 4 (12,800) 38.8, 30.9; on 128 elements p = 3 0.45, 0.56 and
-// p = 4 0.77, 0.85; 3D p = 2 and 3 always the other way.
+// small_elements() draws the line, in elements per SM for 2D meshes; measured on 152 SMs (assemble + condense, ms, here and
+// there):
+//   always here: 3D p = 1, 48,000 elements 50.8, 58.6; 2D Euler p = 1 (51,200) 12.4, 12.5, p = 2 (32,768) 12.4, 13.9,
+//     p = 3 (18,432) 14.6, 15.3; 2D NS p = 2 (32,768) 19.9, 21.6
+//   2D NS p = 3, up to seven per SM: 128 elements 0.446, 0.556; 512 0.820, 0.792; 800 1.216, 1.311; 968 1.470, 1.481;
+//     1,058 1.475, 1.513; then 1,152 1.578, 1.548; 1,352 1.831, 1.830; 1,568 2.180, 2.197; 2,048 2.804, 2.640; 18,432
+//     23.1, 22.0
+//   2D NS p = 4, up to one: 128 0.765, 0.852; then 162 1.044, 0.973; 512 2.106, 1.671; 8,192 24.5, 19.5
+//   2D Euler p = 4, up to two: 128 0.511, 0.599; 288 0.696, 0.715; then 338 0.913, 0.905; 512 1.426, 1.297
+//   3D p = 2 and 3: never (6 elements 1.78, 1.68 and 7.95, 4.37; 3,072 24.7, 16.0 and 167.6, 67.5)
+// The two sides round differently: an element's blocks may differ in the last bits between meshes on either side.
 #pragma once
 #include "assemble_fp64.cuh"
 #include "ctx.hpp"
@@ -16,8 +23,9 @@ namespace small {
 template <class C>
 constexpr bool kCompiled = C::NV < 40 || C::D == 2;  // configurations that can take these kernels
 template <class C>
-bool small_elements(int64_t E) {
-  return C::NV < 40 || (!C::VISC && C::NV == 40) || (C::D == 2 && E <= 304);
+bool small_elements(int64_t E, int num_sms) {
+  constexpr int per_sm = C::NV == 40 ? 7 : C::VISC ? 1 : 2;
+  return C::NV < 40 || (!C::VISC && C::NV == 40) || (C::D == 2 && E <= per_sm * (int64_t)num_sms);
 }
 
 // doubles per volume and face point

@@ -58,3 +58,24 @@ def test_elements_past_the_small_mesh_rule_match_oracle(p):
             assert rel_fro(S[e], ref["S"]) <= 1e-10
             assert rel_fro(g[e], ref["g"]) <= 1e-10
             assert rel_fro(rec[e, :nv * nt].reshape(nv, nt), ref["X"][Q[e].size:]) <= 1e-10
+
+
+@pytest.mark.parametrize("reynolds,p,sizes", [(500.0, 3, (23, 24)), (500.0, 4, (8, 9)), (0.0, 4, (12, 13))])
+def test_both_sides_of_the_small_mesh_lines_match_oracle(reynolds, p, sizes):
+    """The lines lie at seven, one and two elements per SM (1,064, 152 and 304 on 152 SMs)."""
+    for n in sizes:
+        case = Case(f"2d_p{p}", 2, n, p, 1.25 * n, 0.5, reynolds, 0.71, "vortex")
+        prob, Q, V, Vh = oracle_setup(case)
+        gc = GpuCase(case)
+        gc.assemble(gc.history())
+        assert int(gc.status.abs().sum()) == 0
+        nv, nt = gc.info["nv"], gc.info["nt"]
+        for e in (0, 1, gc.info["n_elem"] - 1):
+            q = None if Q is None else Q[e]
+            nq = 0 if q is None else q.size
+            he = prob.history_weak(e, [V[e] * (1 + 1e-3)], [case.mass_coef])
+            ref = prob.condense(e, q, V[e], prob.gather_trace(Vh, e), case.mass_coef, he)
+            assert rel_fro(gc.S[e].cpu().numpy(), ref["S"]) <= 1e-10
+            assert rel_fro(gc.g[e].cpu().numpy(), ref["g"]) <= 1e-10
+            X = gc.recov[e, :nv * nt].cpu().numpy().reshape(nv, nt)
+            assert rel_fro(X, ref["X"][nq:]) <= 1e-10
