@@ -77,8 +77,8 @@ enum { HDG_SCHEME_HDG = 0, HDG_SCHEME_EDG = 1, HDG_SCHEME_IEDG = 2 };
  *                tolerance (left set only when the FP64 recomputation is switched off)
  *   FP64         mixed form: the block missed the tolerance (or timed out) and was recomputed
  *                by the FP64 kernels (hdg_ctx_set_refinement); S, g, X, y are the FP64 form's
- *   TIMEOUT      mixed form, tcgen05 condensation: a bounded wait for its operands or its
- *                tensor-core products gave up (about a second); the kernel freed its tensor
+ *   TIMEOUT      mixed form, tcgen05 kernels: a bounded wait for operands or tensor-core
+ *                products gave up (about a second); the kernel freed its tensor
  *                memory and returned, the context stays usable, and the block's outputs are
  *                invalid unless the FP64 recomputation replaced them (then FP64 is set instead) */
 enum { HDG_ELEM_NONPHYSICAL = 1, HDG_ELEM_SINGULAR = 2, HDG_ELEM_REFINE = 4, HDG_ELEM_FP64 = 8,

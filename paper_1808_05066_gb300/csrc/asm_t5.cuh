@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
       uint32_t a_use = 0, a_seen = 0;  // per slot: parity of its next "empty" wait; whether it was used before
       int w = 0, w_par = 1, nw = 0;
       uint32_t a_out = 0;              // per slot: loads issued, modulo 2 (for the drain)
-      bool ok = true;
+      bool ok = true, stall = (a.stall_first_copy & kStallAssembly) && blockIdx.x == 0;
       for (int t = first; t < ntile && ok; t += stride) {
         const bool p0 = t < P0.ntile;
         const T5Prog& P = p0 ? P0 : P1;
@@ -411,7 +411,8 @@ __global__ void __launch_bounds__(kT5Threads, 1) k_asm_t5(AssembleArgs a, T5Prog
               if (!ok) break;
               a_seen |= 1u << k;
               mbar_arrive_expect_tx(a_full + k, ASTEP);
-              bulk_g2s(As + (size_t)k * ASTEP, Ts + (int64_t)(s0 + k) * ASTEP, ASTEP, a_full + k);
+              if (!stall) bulk_g2s(As + (size_t)k * ASTEP, Ts + (int64_t)(s0 + k) * ASTEP, ASTEP, a_full + k);
+              stall = false;  // the test hook leaves the first copy's phase incomplete
               a_out ^= 1u << k;
             }
           }

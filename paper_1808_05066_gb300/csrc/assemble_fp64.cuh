@@ -53,9 +53,10 @@ struct AssembleArgs {
   // replaces the flag by HDG_STATUS_FP64 (the block is now the FP64 form's).
   int only_flag;
   float refine_tol;     // mixed condensation: tolerance of the refinement status bit
-  int stall_first_copy; // test hook of k_condense_t5: its first operand copy is never issued
+  int stall_first_copy; // test hooks (kStall*): the kernel never issues its first operand copy
 };
 
+enum { kStallCondense = 1, kStallAssembly = 2 };  // k_condense_t5; the first CTA of k_asm_t5
 enum { HDG_STATUS_NONPHYSICAL = 1, HDG_STATUS_SINGULAR = 2, HDG_STATUS_REFINE = 4, HDG_STATUS_FP64 = 8,
        HDG_STATUS_TIMEOUT = 16 };
 

@@ -425,7 +425,7 @@ int run_mixed(hdg_ctx* ctx, const double* V, const double* Vhat, const double* h
   a.R = R;
   a.status = status;
   a.refine_tol = (float)ctx->refine_tol;
-  a.stall_first_copy = ctx->t5_stall ? 1 : 0;
+  a.stall_first_copy = (ctx->t5_stall ? kStallCondense : 0) | (ctx->asm_stall ? kStallAssembly : 0);
   const int64_t ch = ctx->chunk;
   a.ptv = ctx->d_scr;
   a.ptf = a.ptv + ch * vol;

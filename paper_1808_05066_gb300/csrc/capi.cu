@@ -373,7 +373,13 @@ int hdg_ctx_create(hdg_mesh_t mesh, const hdg_physics* phys, int device, hdg_ctx
     long v = std::strtol(cv, nullptr, 10);
     if (v >= 0 && v < 4) c->cond_variant = (int)v;
   }
-  if (const char* st = std::getenv("HDG_T5_STALL_FIRST_COPY")) c->t5_stall = std::strtol(st, nullptr, 10) != 0;
+  auto env_set = [](const char* name) {
+    const char* v = std::getenv(name);
+    return v && std::strtol(v, nullptr, 10) != 0;
+  };
+  c->t5_stall = env_set("HDG_T5_STALL_FIRST_COPY");
+  c->asm_stall = env_set("HDG_ASM_STALL_FIRST_COPY");
+  c->mv_stall = env_set("HDG_MATVEC_STALL_FIRST_COPY");
   if (const char* sb = std::getenv("HDG_SINK_BUFFERS")) {  // device buffers of the host-sink ring
     long v = std::strtol(sb, nullptr, 10);
     if (v >= 2 && v <= hdg_ctx::kSinkMax) c->sink_bufs = (int)v;
@@ -905,7 +911,7 @@ int hdg_newton_solve(hdg_ctx_t ctx, double* V, double* Vhat, const double* hist,
       return HDG_ERR_SINGULAR;
     }
     if (bits & HDG_ELEM_TIMEOUT) {  // only with the FP64 recomputation switched off
-      set_error("hdg_newton_solve: a bounded wait in the element condensation gave up");
+      set_error("hdg_newton_solve: a bounded wait in the element assembly or condensation gave up");
       return HDG_ERR_TIMEOUT;
     }
     if (bits & HDG_ELEM_REFINE) {  // only with the FP64 recomputation switched off

@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256, 1) k_condense_t5(AssembleArgs a) {
       uint32_t bytes;
       const unsigned char* src = job_src(next_load, &bytes);
       mbar_arrive_expect_tx(full + slot, bytes);
-      if (!(a.stall_first_copy && next_load == 0))  // the test hook leaves this phase incomplete
+      if (!((a.stall_first_copy & kStallCondense) && next_load == 0))  // the test hook leaves this phase incomplete
         bulk_g2s(As + (size_t)slot * OZS * TILE, src, bytes, full + slot);
       ++next_load;
     }

@@ -416,7 +416,8 @@ __global__ void __launch_bounds__(CondTC<C, 256, OZS>::PTH) k_condense_prep(Asse
   const bool ok = gj_inverse_reg<NV, LDA, PTH>(G, gsi, prow);
   float* ai = pre + Q::PREP_AI;
   for (int t = tid; t < NV * LDA; t += PTH) ai[t] = (t % LDA) < NV ? G[t] : 0.f;
-  if (tid == 0 && !ok) atomicOr(a.status + e, HDG_STATUS_SINGULAR);
+  // blocks whose assembly gave up a wait are no statement about the element: they are recomputed or reported as such
+  if (tid == 0 && !ok && !(a.status[e] & HDG_STATUS_TIMEOUT)) atomicOr(a.status + e, HDG_STATUS_SINGULAR);
 }
 
 template <class C, int NTHREADS, int OZS>
