@@ -295,15 +295,8 @@ HDG_DEVI void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// mbar_wait without sleeping between the first polls: these waits last a microsecond or less
-HDG_DEVI bool t5_wait(uint64_t* bar, uint32_t parity) {
-  constexpr int LIMIT = 1 << 22;
-  for (int i = 0; i < LIMIT; ++i) {
-    if (mbar_try(bar, parity)) return true;
-    if (i > 4096) __nanosleep(256);
-  }
-  return false;
-}
+// these waits last a microsecond or less: no sleep between the first polls
+HDG_DEVI bool t5_wait(uint64_t* bar, uint32_t parity) { return mbar_wait(bar, parity, 4096); }
 
 // The sum of the diagonals, sum_d 2^(-8 d) Q_d, as a normalised double-float. Every Q_d is an integer below 2^24,
 // so the two pairs (Q0, Q1), (Q2, Q3) and their sum are exact two-term sums by an FMA and its residual

@@ -174,7 +174,6 @@ __global__ void __launch_bounds__(256, 1) k_condense_t5(AssembleArgs a) {
   constexpr int NSLOT = Q::NSLOT, NTH = Q::NTH, NWARP = NTH / 32, LDA = Q::LDA;
   constexpr uint32_t TILE = Q::TILE, BTILE = Q::BTILE;
   constexpr uint32_t IDESC = UmmaIdesc<128, NB>::value;
-  constexpr int WAIT = 1 << 22;  // polls of a bounded wait (about a second with the back-off)
   static_assert(LDA == P::LDA, "prep layout");
   extern __shared__ __align__(128) unsigned char smem_t5[];
   unsigned char* As = smem_t5;                                            // [NSLOT][OZS][TILE]
@@ -257,7 +256,7 @@ __global__ void __launch_bounds__(256, 1) k_condense_t5(AssembleArgs a) {
   auto produce = [&]() {
     while (next_load < njobs && next_load < issued + NSLOT - 1) {
       const int slot = next_load % NSLOT, use = next_load / NSLOT;
-      if (use > 0 && !mbar_wait(empty + slot, (use - 1) & 1, WAIT)) {
+      if (use > 0 && !mbar_wait(empty + slot, (use - 1) & 1)) {
         s_fail = 1;
         return;
       }
@@ -273,7 +272,7 @@ __global__ void __launch_bounds__(256, 1) k_condense_t5(AssembleArgs a) {
   // of `tile` (columns acc0 + d NB); npair products with s + t < nsl
   auto issue = [&](int J, int nsl, uint32_t acc0, int kt) {
     const int slot = J % NSLOT;
-    if (s_fail || !mbar_wait(full + slot, (J / NSLOT) & 1, WAIT)) {
+    if (s_fail || !mbar_wait(full + slot, (J / NSLOT) & 1)) {
       s_fail = 1;
       return;
     }
@@ -293,7 +292,7 @@ __global__ void __launch_bounds__(256, 1) k_condense_t5(AssembleArgs a) {
       umma_commit(accb);
       produce();  // the next phase's first operands, meanwhile
     }
-    const bool ok = mbar_wait(accb, acc_phase & 1, WAIT);
+    const bool ok = mbar_wait(accb, acc_phase & 1);
     ++acc_phase;
     if (!ok) s_fail = 1;
     tc_fence_after();
@@ -524,10 +523,10 @@ __global__ void __launch_bounds__(256, 1) k_condense_t5(AssembleArgs a) {
   }
   // drain: every copy issued has landed and every MMA has completed before TMEM is freed
   if (tid == 0) {
-    for (int J = issued; J < next_load; ++J) mbar_wait(full + J % NSLOT, (J / NSLOT) & 1, WAIT);
+    for (int J = issued; J < next_load; ++J) mbar_wait(full + J % NSLOT, (J / NSLOT) & 1);
     umma_commit(accb);
   }
-  mbar_wait(accb, acc_phase & 1, WAIT);
+  mbar_wait(accb, acc_phase & 1);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {

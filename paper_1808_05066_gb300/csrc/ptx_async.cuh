@@ -23,11 +23,24 @@ HDG_DEVI bool mbar_try(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Waits for the phase of the given parity to complete; gives up after `limit` polls.
-HDG_DEVI bool mbar_wait(uint64_t* bar, uint32_t parity, int limit) {
-  for (int i = 0; i < limit; ++i) {
+HDG_DEVI unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// Waits for the phase of the given parity to complete: `spins` polls, then polls 256 ns apart; gives up after a
+// second. The limit is a time because a poll that fails may itself suspend the thread for microseconds (4M polls
+// took 4 to 16 s); the number of polls is bounded as well, and some follow the deadline, in case the
+// kernel was not running meanwhile.
+constexpr unsigned long long kWaitNs = 1000000000ull;
+HDG_DEVI bool mbar_wait(uint64_t* bar, uint32_t parity, int spins = 64) {
+  for (int i = 0; i < spins; ++i)
     if (mbar_try(bar, parity)) return true;
-    if (i > 64) __nanosleep(256);
+  const unsigned long long t0 = global_ns();
+  for (int i = 0, late = 0; i < 1 << 22 && late < 64; ++i) {
+    if (mbar_try(bar, parity)) return true;
+    __nanosleep(256);
+    if (global_ns() - t0 > kWaitNs) ++late;
   }
   return false;
 }

@@ -255,7 +255,6 @@ __global__ void k_elem_matvec_df(const df2* S, const double* x, const int* tgidx
 // HBM bound; 3D p = 3, 3,072 elements (0.98 GB): 170 us, against 298 us with chunks shared by the
 // warps of a CTA and 353 us by rows_times_vector.
 constexpr int kMvRows = 8, kMvWarps = 8, kMvMaxSlots = 4;
-constexpr int kMvWaitPolls = 4 * 1000 * 1000;  // ~1 s at 256 ns per poll
 __global__ void __launch_bounds__(32 * kMvWarps) k_elem_matvec_ring(const df2* __restrict__ Sdf, const double* x,
                                                                    const int* tgidx, int64_t E, int NT, int M, int slots,
                                                                    double* w, int* err, const int* skip, bool stall) {
@@ -292,13 +291,13 @@ __global__ void __launch_bounds__(32 * kMvWarps) k_elem_matvec_ring(const df2* _
       cur = e;
       __syncwarp();
     }
-    const bool ok = mbar_wait(full + slot, (uint32_t)(((q - q0) / slots) & 1), kMvWaitPolls);
+    const bool ok = mbar_wait(full + slot, (uint32_t)(((q - q0) / slots) & 1));
     if (!__all_sync(0xffffffffu, ok)) {
       if (lane < rows) w[e * NT + k * kMvRows + lane] = __longlong_as_double(0x7ff8000000000000LL);
       if (lane == 0) {
         atomicExch(err, 1);
         for (int64_t p = q; p < q1 && p < q + slots; ++p)
-          mbar_wait(full + (p - q0) % slots, (uint32_t)(((p - q0) / slots) & 1), kMvWaitPolls);
+          mbar_wait(full + (p - q0) % slots, (uint32_t)(((p - q0) / slots) & 1));
       }
       return;
     }

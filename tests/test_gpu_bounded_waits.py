@@ -1,6 +1,8 @@
 """The bounded waits of the streaming kernels, run out on purpose: a hook makes the host ask for a first operand copy that
 is never issued, the kernel gives up after about a second a wait, drains its other copies, reports and returns. Nothing
 faults, and the context stays usable."""
+import time
+
 import pytest
 
 from hdg_cases import CASES, GpuCase
@@ -67,3 +69,22 @@ def test_trace_product(monkeypatch):
     free = GpuCase(case)
     it, res = hdg.hdg_trace_solve(free.ctx.handle, gc.S, gc.g, x, hdg.HDG_SOLVER_GMRES, 1e-10, 600)
     assert it > 1 and res <= 1e-10
+
+
+@pytest.mark.parametrize("hook", ["HDG_ASM_STALL_FIRST_COPY", "HDG_MATVEC_STALL_FIRST_COPY"])
+def test_waits_last_about_a_second(hook, monkeypatch):
+    """Two waits in a row run out (the operand's and its drain's): two seconds, and three to launch and return."""
+    monkeypatch.setenv("HDG_COND_VARIANT", "2")
+    GpuCase(CASES["ns3d_p2"]).assemble(None, precision=1)   # kernels are loaded
+    monkeypatch.setenv(hook, "1")
+    gc = GpuCase(CASES["ns3d_p2"])
+    hdg = gc.hdg
+    gc.assemble(gc.history())
+    x = gc.torch.empty_like(gc.Vhat)
+    t = time.monotonic()
+    if "ASM" in hook:
+        gc.assemble(gc.history(), precision=1)
+        assert (gc.status == hdg.HDG_ELEM_FP64).any()
+    else:
+        _code(lambda: hdg.hdg_trace_solve(gc.ctx.handle, gc.S, gc.g, x, hdg.HDG_SOLVER_GMRES, 1e-10, 1))
+    assert 0.9 < time.monotonic() - t < 5.0
