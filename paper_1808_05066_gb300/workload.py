@@ -114,25 +114,34 @@ def bench_workload_name() -> str:
     return "ns3d_p3_tgv"
 
 
+def _contraction_macs(D, M, viscous, NP, NG, NTN, NGF, own):
+    """Multiply-adds of the FP64 contraction of one element (element_fp64.cuh): NTN trace nodes on
+    all faces, `own` the sum over the faces of their trace nodes squared. Per pair (i, l): the trial
+    side at the face points, the faces' rows, the left factors and products of the value operator
+    and, for the (M - 1)^2 pairs with a viscous part, of the D gradient operators (interior columns)
+    and of the D + 1 that meet one face's trace columns each."""
+    NF = D + 1
+    value = NF * NGF * NP + NTN * NGF + NTN * NGF * NP + own * NGF + NP * NG * (1 + D) + NP * NP * NG
+    grad = (NF * NGF * (D * NP + NTN) + (NTN * NTN - own) * NGF + NF * NP * NG * D + D * NP * NP * NG + NP * NTN * NG)
+    return M * M * value + ((M - 1) ** 2 * grad if viscous else 0)
+
+
+def _condensation_macs(NV, NT):
+    """LU, solves for X and y, Schur product and g."""
+    return NV ** 3 / 3.0 + (NT + 1) * NV ** 2 + NT * NT * NV + NT * NV
+
+
 def flops_per_element(info: dict, viscous: bool, kernel: str) -> float:
-    """Useful floating-point operations per element of the FP64 form, counted from the
-    loop structure of the kernels (multiply + add = 2 flops):
-      assemble: volume contraction per (i, l): NP x [NP x ng x NR + NT' x ng x (NR-1)]
-                + the left factor NP x ng x NR x (D+1); face contraction per face and (i, l):
-                NFN x NZ x NGF x NRF + NFN x NGF x NRF;
-      condense: LU NV^3/3 + solves (NT + 1) NV^2 + Schur NT^2 NV + NT NV."""
-    D, M = info["dim"], info["m"]
-    NP, NFN, NF, NG, NGF = info["Np"], info["Nf"], info["nF"], info["NG"], info["NGF"]
-    NV, NT = info["nv"], info["nt"]
-    NZ = NP + NF * NFN
-    NR = D + 1 if viscous else 1
-    NRF = D + 2 if viscous else 2
+    """Useful floating-point operations per element of the FP64 form (multiply + add = 2 flops), as the
+    kernels of element_fp64.cuh count them, without the padding of their tiles: "assemble" the
+    contraction, "condense" the factorisation, solves and Schur product. (The kernels for small
+    elements contract in physical coordinates and take more for the same blocks.)"""
+    NFN, NF = info["Nf"], info["nF"]
     if kernel == "assemble":
-        vol = M * M * (NP * (NP * NG * NR + NF * NFN * NG * (NR - 1)) + NP * NG * NR * (D + 1))
-        face = NF * M * M * (NFN * NZ * NGF * NRF + NFN * NGF * NRF)
-        return 2.0 * (vol + face)
+        return 2.0 * _contraction_macs(info["dim"], info["m"], viscous, info["Np"], info["NG"], NF * NFN, info["NGF"],
+                                       NF * NFN * NFN)
     if kernel == "condense":
-        return 2.0 * (NV ** 3 / 3.0 + (NT + 1) * NV ** 2 + NT * NT * NV + NT * NV)
+        return 2.0 * _condensation_macs(info["nv"], info["nt"])
     raise ValueError(kernel)
 
 
@@ -142,22 +151,14 @@ FP64_PIPE_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 
 def class_flops_per_element(pk: int, pt: int, nt_own: int) -> float:
-    """FP64 flops of one element of the mixed-degree fused kernel (3D Navier-Stokes), counted from
-    its loops like flops_per_element: element degree pk (volume rule pk + 1), trace degree pt on
-    every face (face rule pt + 1), the face contractions over the element's face nodes (degree pk)
-    and the trace nodes (degree pt), and the condensation with the element's own trace size
-    nt_own; the projection onto the faces' own spaces is not counted."""
+    """FP64 flops of one element of the mixed-degree fused kernel (3D Navier-Stokes), counted like
+    flops_per_element: element degree pk (volume rule pk + 1), face rule pt + 1, and nt_own trace
+    unknowns in the faces' own degrees (taken as equal, which counts their products least). The trace
+    prolongation and the combinations at faces of a higher degree are not counted."""
     D, M, NF = 3, 5, 4
-    NP = (pk + 1) * (pk + 2) * (pk + 3) // 6
-    NFK = (pk + 1) * (pk + 2) // 2
-    NFN = (pt + 1) * (pt + 2) // 2
-    NG, NGF = (pk + 1) ** 3, (pt + 1) ** 2
-    NZ, NV = NP + NF * NFN, NP * M
-    NR, NRF = D + 1, D + 2
-    vol = M * M * (NP * (NP * NG * NR + NF * NFN * NG * (NR - 1)) + NP * NG * NR * (D + 1))
-    face = NF * M * M * ((NFK + NFN) * NZ * NGF * NRF + (NFK + NFN) * NGF * NRF)
-    cond = NV ** 3 / 3.0 + (nt_own + 1) * NV ** 2 + nt_own * nt_own * NV + nt_own * NV
-    return 2.0 * (vol + face + cond)
+    NP, NTN = (pk + 1) * (pk + 2) * (pk + 3) // 6, nt_own // M
+    return 2.0 * (_contraction_macs(D, M, True, NP, (pk + 1) ** 3, NTN, (pt + 1) ** 2, NTN * NTN / NF) +
+                  _condensation_macs(NP * M, nt_own))
 
 
 SLICES = 6  # exact bf16 slices per operand in the mixed form's tensor-core products
@@ -168,47 +169,42 @@ def slice_flops_per_element(info: dict, viscous: bool, kernel: str) -> float:
     2 x rows x columns x contraction length of every nonzero operator block, times the
     S(S+1)/2 slice products. Tile padding and products a kernel shape adds are not counted, so
     this never exceeds what a kernel executes:
-      mixed_assemble: volume: rows (i, l, node) = m^2 NP, contraction NG per operator; the value
-                      operator meets the NP interior columns, each of the NR - 1 gradient
-                      operators all NZ; and the faces (one kernel forms both);
-      mixed_face:     the faces' share of it: per face rows m^2 NFN, contraction NGF; value operator
-                      NP columns, trace operator the face's own NFN, each of the NRF - 2
-                      gradient operators all NZ;
+      mixed_assemble: a row per pair (i, l), a column per (test, trial) node pair, k over (operator,
+                      point). Every pair: the value and D gradient tests at the volume points
+                      against the NP interior columns, the faces' value operators against the
+                      nodes on the face and the face's own trace columns. Pairs with a viscous part: D^2
+                      operators against the interior columns and D against every trace column,
+                      and on the faces D against all interior columns, one against every trace column;
       mixed_condense: r0 = B - A' X0 and S = D - C' X: NV + NT rows, NT + 1 right-hand sides,
                       contraction NV."""
     D, M = info["dim"], info["m"]
     NP, NFN, NF, NG, NGF = info["Np"], info["Nf"], info["nF"], info["NG"], info["NGF"]
     NV, NT = info["nv"], info["nt"]
-    NZ = NP + NF * NFN
-    NR = D + 1 if viscous else 1
-    NRF = D + 2 if viscous else 2
+    NTN = NF * NFN
     prod = SLICES * (SLICES + 1) // 2
-    face = 2.0 * prod * NF * (M * M * NFN) * NGF * (NP + NFN + (NRF - 2) * NZ)
     if kernel == "mixed_assemble":
-        return 2.0 * prod * (M * M * NP) * NG * (NP + (NR - 1) * NZ) + face
-    if kernel == "mixed_face":
-        return face
+        macs = M * M * (NP * NP * NG * (1 + D) + 2 * NTN * NFN * NGF)
+        if viscous:
+            macs += (M - 1) ** 2 * (NP * NP * NG * D * D + NP * NTN * NG * D + NTN * NP * NGF * D + NTN * NTN * NGF)
+        return 2.0 * prod * macs
     if kernel == "mixed_condense":
         return 2.0 * prod * (NV + NT) * (NT + 1) * NV
     raise ValueError(kernel)
 
 
-def algorithmic_bytes_per_element(info: dict, kernel: str) -> int:
+def algorithmic_bytes_per_element(info: dict, viscous: bool, kernel: str) -> int:
     """HBM bytes one element needs moved by a mixed-form kernel (8-byte values):
       mixed_assemble: read the point tensors, write A', B', C' and D';
-      mixed_face:     the share of the face point tensors, C' and D';
       mixed_condense: the method's outputs only: write S, X, y and g (the blocks the assembly
                       parks in HBM for it are this implementation's, not the method's)."""
     D, M = info["dim"], info["m"]
-    NP, NFN, NF, NG, NGF = info["Np"], info["Nf"], info["nF"], info["NG"], info["NGF"]
+    NF, NG, NGF = info["nF"], info["NG"], info["NGF"]
     NV, NT = info["nv"], info["nt"]
-    pt_vol = M + D * M + M * M + D * M * M + D * M * M * D
-    pt_face = M + 2 * M * M + M * M * D
-    face = 8 * (NF * NGF * pt_face + NT * (NV + NT))
+    visc = (D + 1) * (M - 1) ** 2 if viscous else 0  # dG/dq per face point; D times that per volume point
+    pt_vol = M + D * M + M * M + D * M * M + D * visc
+    pt_face = M + 2 * M * M + visc
     if kernel == "mixed_assemble":
-        return 8 * (NG * pt_vol + NV * (NV + NT)) + face
-    if kernel == "mixed_face":
-        return face
+        return 8 * (NG * pt_vol + NF * NGF * pt_face + (NV + NT) * (NV + NT))
     if kernel == "mixed_condense":
         return 8 * (NT * NT + NV * NT + NV + NT)
     raise ValueError(kernel)
@@ -216,13 +212,9 @@ def algorithmic_bytes_per_element(info: dict, kernel: str) -> int:
 
 def method_flops_per_element(info: dict, viscous: bool, kernel: str) -> float:
     """The method's own flops per element of a mixed-form kernel, the same count as the FP64
-    form's kernels (flops_per_element): the assembly contractions for mixed_assemble (mixed_face: the
-    faces' share by slice products), the LU, solves and Schur product for mixed_condense."""
-    if kernel == "mixed_condense":
-        return flops_per_element(info, viscous, "condense")
-    asm = flops_per_element(info, viscous, "assemble")
-    return asm * slice_flops_per_element(info, viscous, kernel) / slice_flops_per_element(info, viscous, "mixed_assemble")
-
+    form's kernels (flops_per_element): the contractions for mixed_assemble, the LU, solves and
+    Schur product for mixed_condense."""
+    return flops_per_element(info, viscous, {"mixed_assemble": "assemble", "mixed_condense": "condense"}[kernel])
 
 
 def main(argv=None):
