@@ -19,8 +19,8 @@
 // meets slices 0 .. 5 - s in ONE instruction of N = 32 (6 - s), whose accumulator columns are the diagonals
 // s .. 5: six instructions per 16 entries of k instead of 21.
 //
-// Bound and measurements (82,944 tetrahedra, p = 3; the replaced volume, face and operator kernels: 277 ms):
-// rows 18 ms, products 106 ms, of which the MMAs 57; the rest is the traffic of the running sums and of
+// Bound and measurements (82,944 tetrahedra, p = 3; the replaced volume, face, operator and residual kernels: 277 ms):
+// rows and residuals 23 ms, products 103 to 109 ms from one GPU to another, of which the MMAs 57; the rest is the traffic of the running sums and of
 // the blocks' 8-byte entries (4 MB of DRAM traffic an element).
 //
 // One persistent CTA per SM takes tiles of 128 rows. The tile's slices of one chunk (up to 8 steps of 16

@@ -119,8 +119,8 @@ struct hdg_ctx {
   int newton_solver = HDG_SOLVER_AUTO;
   double newton_rtol = 1e-12;
   int newton_max_it = 600;
-  // dynamic shared-memory limits raised on this context's device (cudaFuncSetAttribute
-  // applies per device; a context belongs to one device)
+  // dynamic shared-memory limits raised on this context's device. A limit belongs to the kernel and the device and all
+  // contexts share it, so every context sets the same value, whatever its own sizes
   bool attr_fp64 = false, attr_mixed = false, attr_noalloc = false, attr_matvec = false;
   int num_sms = 0;               // SMs of the device (persistent grids)
   hdg::PMix* pm = nullptr;       // mixed-degree mesh: class tables, packed layout, work queue
