@@ -194,13 +194,13 @@ def parse():
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per element of the mixed tensor-core
-# kernels from one ncu --set full capture on 3,072 elements; every element is its own CTA (or
-# row blocks of one), so traffic grows with the element count and scales to a launch by its
-# elements. Valid only while the kernel sources hash to the digest they were captured on.
+# kernels from one ncu capture on 1,296 elements (more than L2 holds several times over); traffic
+# grows with the element count and scales to a launch by its elements. Valid only while the kernel
+# sources hash to the digest they were captured on.
 NCU_TRAFFIC = {
-    "source": "profiles/ncu_mixed_kernels_ns3d_p3_n8.md",
-    "sources_sha256": "4f9eda78a7eadb3a5606341f4b5fa50b2b5a5f71e103193bc010daf658212a7a",
-    "bytes_per_element": {"mixed_assemble": 600_747, "mixed_face": 1_255_572, "mixed_condense": 2_617_894},
+    "source": "profiles/ncu_mixed_kernels_ns3d_p3_n6.md",
+    "sources_sha256": "5ab3f99d2cf46a6a3abc049d5255352aa8f21e36f33d58df059bbc6bdbbeb8fc",
+    "bytes_per_element": {"mixed_assemble": 3_988_032, "mixed_condense": 1_390_173},
 }
 
 # the sources that define the captured kernels and their launch shapes (device code and the
